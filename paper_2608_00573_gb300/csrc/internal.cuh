@@ -291,7 +291,9 @@ cudaError_t launch_watchdog_selftest(int* err, uint64_t limit_ns, cudaStream_t s
 // visible before touching anything written upstream.  Single-wave and
 // persistent kernels let the next grid be scheduled right after their wait
 // (pdl_trigger), multi-wave kernels only when each block is done, so that
-// waiting blocks never take the room of their later waves.  After a launch
+// waiting blocks never take the room of their later waves, and the single-CTA
+// GEMM when its last loads are issued (waiting GEMM CTAs would keep other
+// streams off the SMs).  After a launch
 // without the attribute pdl_wait returns at once.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
