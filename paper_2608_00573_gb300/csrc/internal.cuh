@@ -61,7 +61,7 @@ struct DevTables {
     int max_layer_cand;      // largest number of candidates of one layer
     const float* trans;      // [M][M]
     const float* comp;       // [N][M]
-    const float* P;          // [N-1][E][E]
+    const float* PT;         // [N-1][E][E] P_l(k -> k') with k' the slow index
     const float* theta;      // [N]
     const float* lambda;     // [N]
     const float* eps;        // [N]

@@ -193,7 +193,7 @@ struct trimmoe {
     size_t rows_part = 0;             // max over T <= T_max of ksplit(T) * T
     float* ctab = nullptr;
     int max_layer_cand = 1;
-    float *trans = nullptr, *comp = nullptr, *P = nullptr, *theta = nullptr, *lambda = nullptr, *eps = nullptr;
+    float *trans = nullptr, *comp = nullptr, *PT = nullptr, *theta = nullptr, *lambda = nullptr, *eps = nullptr;
 
     // workspaces
     int32_t* topk_idx = nullptr;
@@ -663,7 +663,7 @@ extern "C" trimmoe_status trimmoe_create(const trimmoe_config* cfg, const trimmo
               h->dalloc(&h->cnorm, cn.size()) && h->dalloc(&h->lhat, lh.size()) &&
               h->dalloc(&h->zbuf, h->rows_part * (size_t)n_out) && h->dalloc(&h->sqbuf, h->rows_part) &&
               h->dalloc(&h->trans, (size_t)M * M) && h->dalloc(&h->comp, (size_t)N * M) &&
-              h->dalloc(&h->P, (size_t)std::max(N - 1, 1) * E * E) && h->dalloc(&h->theta, N) &&
+              h->dalloc(&h->PT, (size_t)std::max(N - 1, 1) * E * E) && h->dalloc(&h->theta, N) &&
               h->dalloc(&h->lambda, N) && h->dalloc(&h->eps, N) && h->dalloc(&h->topk_idx, TK) &&
               h->dalloc(&h->topk_g, TK) && h->dalloc(&h->I, T) && h->dalloc(&h->xi, T) &&
               h->dalloc(&h->action, T) && h->dalloc(&h->exp_sel, TK) && h->dalloc(&h->srv_sel, TK) &&
@@ -711,7 +711,14 @@ extern "C" trimmoe_status trimmoe_create(const trimmoe_config* cfg, const trimmo
     up(h->lhat, lh.data(), lh.size() * 2);
     up(h->trans, tab->trans_ms, (size_t)M * M * 4);
     up(h->comp, tab->comp_ms, (size_t)N * M * 4);
-    if (N > 1) up(h->P, tab->P, (size_t)(N - 1) * E * E * 4);
+    if (N > 1) {
+        std::vector<float> pt((size_t)(N - 1) * E * E);
+        for (int l = 0; l + 1 < N; ++l)
+            for (int k = 0; k < E; ++k)
+                for (int kp = 0; kp < E; ++kp)
+                    pt[((size_t)l * E + kp) * E + k] = tab->P[((size_t)l * E + k) * E + kp];
+        up(h->PT, pt.data(), pt.size() * 4);
+    }
     up(h->theta, tab->theta, N * 4);
     up(h->lambda, tab->lambda, N * 4);
     up(h->eps, tab->eps, N * 4);
@@ -1022,7 +1029,7 @@ static trimmoe_status layer_step_impl(trimmoe_handle h, int layer, int T, trimmo
     dp.tab.max_layer_cand = h->max_layer_cand;
     dp.tab.trans = h->trans;
     dp.tab.comp = h->comp;
-    dp.tab.P = h->P;
+    dp.tab.PT = h->PT;
     dp.tab.theta = h->theta;
     dp.tab.lambda = h->lambda;
     dp.tab.eps = h->eps;
@@ -1267,7 +1274,7 @@ static bool build_all_tables(trimmoe_handle h, int T, const trimmoe_tokens* tok,
     dp.tab.cand_off = h->cand_off;
     dp.tab.ctab = h->ctab;
     dp.tab.max_layer_cand = h->max_layer_cand;
-    dp.tab.P = h->P;
+    dp.tab.PT = h->PT;
     dp.tab.eps = h->eps;
     *err = h->timed(K_DECIDE, st, [&] {
         return launch_lookahead_all(dp, h->la_layers, c.N, h->la_max_thr, h->la_max_depth, st);
