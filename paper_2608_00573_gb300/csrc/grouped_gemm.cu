@@ -39,8 +39,8 @@
 // covers 256 rows of one group (the odd CTA's rows may lie past the group:
 // loaded, computed and masked).
 //
-// Transposed pair variant (routed down projections, ReLU up projections): the
-// weights on the MMA's M side and the tokens on its N side, N rounded up to 16
+// Transposed pair variant (routed down projections, ReLU up projections, SwiGLU
+// up projections of long K): the weights on the MMA's M side and the tokens on its N side, N rounded up to 16
 // per tile, so a group's tail pads at most 15 tokens; described at the kernel.
 //
 // Both pair variants take their tiles in the order above; for long K they
@@ -738,15 +738,19 @@ grouped_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
 // features of a token straight from registers as one 64-byte segment; for
 // short K the epilogue is on the critical path and the results are staged in
 // shared memory and stored as 16-byte pieces of the tokens' rows.
-// SwiGLU stays on the kernels above: its gate and up accumulators would sit
-// in different warps' TMEM lanes, and every way of bringing them together
-// that was tried (through shared memory, or 16-row weight boxes that pair
-// them within a warp) was slower than the padding it saves.
+// SwiGLU: each CTA stages 64 gate rows and the 64 matching up rows, so its TMEM
+// lanes 0-63 are gates and 64-127 their ups, and the two warps that hold the
+// same 32 features swap halves of every 32 tokens through shared memory (fp32,
+// 128 KB a tile: at K = 4096 about 3 % of what the MMAs move, hidden by the main
+// loop; at K = 2048 the swap shows and the row kernels stay ahead).  Against
+// the single-CTA kernel at 330 rows per group: one box instead of 17 % padded
+// rows, Mixtral-shaped layer of 1500 tokens 846 -> 791 us.
 constexpr int kStageBf16 = 32 * 128;           // one 32-token x 128-feature bf16 staging buffer
 constexpr size_t kPairTailBytes = (sizeof(PairSmemTail) + 15) & ~(size_t)15;
 constexpr size_t kPairTSmemBytes = 1024 + (size_t)P_STAGES * P_STAGE_BYTES + kPairTailBytes +
                                    2 * kStageBf16 * sizeof(__nv_bfloat16);
 constexpr int kEpiBar = 1;                    // named barrier of the four epilogue warps
+constexpr int kSwapBar = 2;                   // ... and two of pairs of them (SwiGLU)
 // Store / ReLU epilogues stage their results in shared memory up to this K
 // (the launcher passes the choice as `staged`).  At K = 14336 (the
 // Mixtral-shaped down projection) staged and direct stores measured the same
@@ -779,7 +783,7 @@ __device__ __forceinline__ int tile_tokens(const Tail* tl, int g, int mt) {
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 grouped_gemm_pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW,
-                           const int* __restrict__ goff,
+                           const __grid_constant__ CUtensorMap tmGU, const int* __restrict__ goff,
                            int first_group, int ngroups, int x_rebase, int out_rebase, int K, int n_ft,
                            int w_rows_per_group, int epi_mode, __nv_bfloat16* __restrict__ out, int ldo,
                            int* err, int mblk, int staged, int* __restrict__ sched) {
@@ -811,7 +815,7 @@ grouped_gemm_pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid
         init_tile_queue_bars(tl->tq_full, tl->tq_empty);
         fence_barrier_init();
         prefetch_tmap(&tmX);
-        prefetch_tmap(&tmW);
+        prefetch_tmap(epi_mode == EPI_SWIGLU ? &tmGU : &tmW);
     }
     if (warp == 0) tmem_alloc_pair(smem_u32(&tl->tmem_base), TMEM_COLS);
     tc_fence_before();
@@ -852,7 +856,10 @@ grouped_gemm_pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid
                         break;
                     if (rank == 0) mbar_arrive_expect_tx(smem_u32(&tl->full[s]), 2 * P_STAGE_BYTES);
                     const uint32_t fb = mapa_shared(smem_u32(&tl->full[s]), 0);
-                    tma_load_2d_pair(sW + s * A_BYTES, &tmW, kb * BK, wrow + (int)rank * BM, fb);
+                    if (epi_mode == EPI_SWIGLU)
+                        tma_load_4d_pair(sW + s * A_BYTES, &tmGU, kb * BK, (int)rank * (BM / 2), 0, wrow / (2 * BM), fb);
+                    else
+                        tma_load_2d_pair(sW + s * A_BYTES, &tmW, kb * BK, wrow + (int)rank * BM, fb);
                     tma_load_2d_pair(sX + s * PB_BYTES, &tmX, kb * BK, xrow, fb);
                 }
             }
@@ -924,7 +931,38 @@ grouped_gemm_pair_t_kernel(const __grid_constant__ CUtensorMap tmX, const __grid
             if (!bar_and_named(kEpiBar, 128, ok)) break;
             tc_fence_after();
             const uint32_t tb = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * BN);
-            if (!staged) {
+            if (epi_mode == EPI_SWIGLU) {
+                // Lanes 0-63 hold the gates of this CTA's 64 features, lanes 64-127
+                // their ups: warps q and q ^ 2 hold the same 32 features.  Of each 32
+                // tokens they swap halves through shared memory, so that the gate warp
+                // finishes tokens 0-15 and the up warp tokens 16-31.
+                float* swap = reinterpret_cast<float*>(stage_out);
+                const bool is_up = q >= 2;
+                const int mine = is_up ? 16 : 0;
+                __nv_bfloat16* ocol = out + (size_t)ft * BM + (size_t)rank * (BM / 2) + (q & 1) * 32 + lane;
+#pragma unroll 1
+                for (int c = 0; c < nch; ++c, ++chunk) {
+                    float* buf = swap + (chunk & 1) * (4 * 16 * 32);
+                    uint32_t r[32];
+                    tmem_ld_32x32(tb + c * 32, r);
+                    tmem_ld_wait();
+                    float keep[16];
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) {
+                        keep[j] = __uint_as_float(is_up ? r[16 + j] : r[j]);
+                        buf[(q * 16 + j) * 32 + lane] = __uint_as_float(is_up ? r[j] : r[16 + j]);
+                    }
+                    bar_sync_named(kSwapBar + (q & 1), 64);
+                    const float* other = buf + ((q ^ 2) * 16) * 32 + lane;
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) {
+                        const float got = other[j * 32];
+                        const float gt = is_up ? got : keep[j], up = is_up ? keep[j] : got;
+                        const int tok = c * 32 + mine + j;
+                        if (tok < rows) ocol[(orow + tok) * ldo] = __float2bfloat16_rn(gt / (1.f + __expf(-gt)) * up);
+                    }
+                }
+            } else if (!staged) {
                 // Long K: the main loop hides the epilogue, and shared-memory
                 // traffic would compete with the MMA operand reads, so each
                 // warp stores its 32 features of a token as one 64-byte segment.
@@ -1045,7 +1083,8 @@ cudaError_t launch_grouped_gemm(const GemmLaunch& g, int num_sms, cudaStream_t s
     // a block stays resident while the weight tiles stream past it.
     const long long a_tile_bytes = (long long)BM * g.K * 2;
     if (g.transposed && g.tmB_pair && g.ksplit <= 1 && pair_t_clusters(num_sms) > 0) {
-        if (g.epi_mode != EPI_STORE && g.epi_mode != EPI_RELU) return cudaErrorInvalidValue;
+        if (g.epi_mode != EPI_STORE && g.epi_mode != EPI_RELU && g.epi_mode != EPI_SWIGLU) return cudaErrorInvalidValue;
+        if (g.epi_mode == EPI_SWIGLU && !g.tmB_gu) return cudaErrorInvalidValue;
         // Token-tile blocks of about 64 MB of activations: at K = 14336 eight
         // token tiles, so a round of 76 tiles spans ~9.5 feature tiles x 8 token
         // tiles, close to the square that streams the fewest operand slices
@@ -1053,8 +1092,8 @@ cudaError_t launch_grouped_gemm(const GemmLaunch& g, int num_sms, cudaStream_t s
         const int mblk2 = (int)std::max(1LL, (64LL << 20) / (2 * a_tile_bytes));
         const cudaError_t e = launch_pdl(
             grouped_gemm_pair_t_kernel, dim3(2 * pair_t_clusters(num_sms)), dim3(kThreads), kPairTSmemBytes, st,
-            *g.tmA, *g.tmB_pair, g.goff, g.first_group, g.ngroups, g.a_rebase, g.out_rebase, g.K, g.n_tiles_n,
-            g.b_rows_per_group, g.epi_mode, g.out, g.ldo, g.err, mblk2,
+            *g.tmA, *g.tmB_pair, g.tmB_gu ? *g.tmB_gu : *g.tmB_pair, g.goff, g.first_group, g.ngroups, g.a_rebase,
+            g.out_rebase, g.K, g.n_tiles_n, g.b_rows_per_group, g.epi_mode, g.out, g.ldo, g.err, mblk2,
             g.K <= kStagedMaxK ? 1 : 0, g.sched);
         if (e != cudaSuccess) return e;
         return cudaGetLastError();

@@ -165,8 +165,11 @@ struct GemmLaunch {
     const CUtensorMap* tmB_pair;
     // Non-zero (with tmB_pair): run the transposed pair kernel instead, the
     // weights on the M side of the MMA and the group's tokens on the N side
-    // (STORE or RELU epilogues; ksplit <= 1).
+    // (STORE, RELU or SWIGLU epilogues; ksplit <= 1).
     int transposed;
+    // Transposed SwiGLU launches: the weights in boxes of two runs of 64 rows, 128
+    // apart (a CTA's gate rows and the matching up rows).
+    const CUtensorMap* tmB_gu;
     const int* goff;
     int first_group, ngroups, a_rebase, out_rebase;
     int K, n_tiles_n, b_rows_per_group, epi_mode;
@@ -493,6 +496,15 @@ __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap
         "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"
         " [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
         "l"(reinterpret_cast<uint64_t>(tm)), "r"(x), "r"(y), "r"(bar_cluster)
+        : "memory");
+}
+
+__device__ __forceinline__ void tma_load_4d_pair(uint32_t dst, const CUtensorMap* tm, int c0, int c1, int c2, int c3,
+                                                 uint32_t bar_cluster) {
+    asm volatile(
+        "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(tm)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(bar_cluster)
         : "memory");
 }
 

@@ -57,6 +57,21 @@ bool make_tmap(CUtensorMap* tm, const void* base, uint64_t inner, uint64_t outer
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// SwiGLU up projections [rows][inner], gate and up rows interleaved by kGateUp,
+// as [block][2][kGateUp][inner]; a box is 64 gate rows and the matching up rows
+// of one k-block.
+bool make_tmap_gu(CUtensorMap* tm, const void* base, uint64_t inner, uint64_t rows) {
+    EncodeTiledFn fn = encode_fn();
+    if (!fn) return false;
+    cuuint64_t dims[4] = {inner, kGateUp, 2, rows / (2 * kGateUp)};
+    cuuint64_t strides[3] = {inner * 2, kGateUp * inner * 2, 2 * kGateUp * inner * 2};
+    cuuint32_t box[4] = {64, 64, 2, 1};
+    cuuint32_t es[4] = {1, 1, 1, 1};
+    return fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, es,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // Small batches: routed GEMMs with at most kSplitKRows executed pairs may split K.
 constexpr int kSplitKMax = 8, kSplitKRows = 64;
 // GEMM launches whose groups average at least kPairMinRows rows run on CTA
@@ -71,6 +86,15 @@ inline bool pair_gemm(long long rows_per_group) { return rows_per_group >= kPair
 // weight-streaming bound, and its 256-feature pair tiles would leave a ragged
 // last round (Mixtral-shaped decode at 256 tokens: 15.2 -> 15.6 ms per step).
 constexpr int kTransposedMinRows = 256;
+
+// SwiGLU up projections of those groups run there too from this K on (and below
+// kPairMinRows rows per group, where the row-pair kernel's padding weighs less
+// than the swap of gates and ups): at K = 4096 the Mixtral-shaped layer of 1500
+// tokens (330 rows per group) 838 -> 794 us and the full-block layer of 4200
+// tokens (910 rows) 2085 -> 1997 us against the single-CTA kernel (2030 us on
+// the row-pair kernel); at K = 2048 the main loop is too short to hide the swap
+// (Qwen-shaped layer of 8192 tokens 834 -> 880 us).
+constexpr int kTransposedSwigluMinK = 4096;
 
 // CTA-pair launches with at least this K draw their tiles from a launch-wide
 // counter (a pair whose tiles ran short takes more of them); at shorter K the
@@ -227,6 +251,7 @@ struct trimmoe {
     std::vector<CUtensorMap> tmW13, tmW2, tmW13sh, tmW2sh;
     // the same weights in 128-row boxes (each CTA's half of a B tile in the pair kernel)
     std::vector<CUtensorMap> tmW13p, tmW2p, tmW13shp, tmW2shp;
+    std::vector<CUtensorMap> tmW13gu;     // SwiGLU: runs of 64 gate rows and the matching up rows
 
     // attention sublayer of the full block
     int nqkv = 0;
@@ -754,11 +779,13 @@ extern "C" trimmoe_status trimmoe_create(const trimmoe_config* cfg, const trimmo
     h->tmW13.resize(N);
     h->tmW2.resize(N);
     h->tmW13p.resize(N);
+    h->tmW13gu.resize(N);
     h->tmW2p.resize(N);
     if (has_sh) { h->tmW13sh.resize(N); h->tmW2sh.resize(N); h->tmW13shp.resize(N); h->tmW2shp.resize(N); }
     const __nv_bfloat16* W13 = static_cast<const __nv_bfloat16*>(w->W13);
     const __nv_bfloat16* W2 = static_cast<const __nv_bfloat16*>(w->W2);
     for (int l = 0; l < N && tm; ++l) {
+        if (c.act == 1) tm = make_tmap_gu(&h->tmW13gu[l], W13 + (size_t)l * E * F13 * d, d, (uint64_t)E * F13);
         for (uint32_t box : {256u, 128u}) {
             CUtensorMap* m13 = box == 256 ? &h->tmW13[l] : &h->tmW13p[l];
             CUtensorMap* m2 = box == 256 ? &h->tmW2[l] : &h->tmW2p[l];
@@ -1100,12 +1127,14 @@ static trimmoe_status layer_step_impl(trimmoe_handle h, int layer, int T, trimmo
     // down projection (and the up projection of ReLU experts) runs on the
     // transposed pair kernel, tokens on the MMA's N side so that a group's
     // last tile pads at most 15 tokens; SwiGLU up projections run on the pair
-    // kernel for large groups and the single-CTA kernel otherwise;
+    // kernel for large groups, on the transposed one for middle-sized groups of
+    // long K and on the single-CTA kernel otherwise;
     // decode-sized batches split K on the single-CTA kernel.
     const bool pair_routed = pair_gemm((long long)T * K / E);
     const bool relu = c.act != 1;
     const bool transposed = (long long)T * K / E >= kTransposedMinRows;
-    g1.transposed = relu && transposed;
+    g1.transposed = transposed && (relu || (!pair_routed && d >= kTransposedSwigluMinK));
+    g1.tmB_gu = relu ? nullptr : &h->tmW13gu[layer];
     g1.tmB_pair = (g1.transposed || pair_routed) ? &h->tmW13p[layer] : nullptr;
     g1.goff = h->goff;
     g1.first_group = 0;

@@ -332,6 +332,22 @@ def test_layer_parity_transposed_pair_gemm(name, kw):
     assert tot["exec"] > 0
 
 
+@pytest.mark.parametrize("name,kw", [
+    ("F384_T1100", dict(E=8, k=2, F=384, T=1100, zipf_s=1.0)),
+    ("F128_T515", dict(E=2, k=1, F=128, T=515, zipf_s=0.3)),
+])
+def test_layer_parity_transposed_swiglu(name, kw):
+    """SwiGLU up projections with K = d >= 4096 and groups averaging 256 to 2047
+    rows run on the transposed CTA-pair kernel (gate and up lanes swapped
+    between warps): token tiles from a few rows to 256 with tails inside a
+    16-token step, one and three blocks of 128 features."""
+    cfg = small_cfg(name=name, N=2, d=4096, M=10, H=3, seed=97, **kw)
+    reports = _run_all_layers(cfg, theta=0.9, exit_bias=1.0)
+    tot = {k: sum(r[k] for r in reports) for k in ("exec", "skip", "exit")}
+    print(name, tot, [round(r["max_rel_err"], 5) for r in reports])
+    assert tot["exec"] > 0
+
+
 def test_layer_parity_decision_lane_groups_of_16():
     """8 < E <= 16 with more tokens than the resident warps (T >= 16 x SMs):
     the decision kernel runs two tokens per warp on 16-lane groups."""
