@@ -87,14 +87,54 @@ __device__ __forceinline__ float sum_parts(const float* __restrict__ base, size_
     return acc;
 }
 
-// The same for up to kMS values at once: value u sums base[off + u * ustride]
-// over the n parts (u < nv), parts in index order.  Every load of one part is
-// issued before the additions.
+// NP such sums at once (base[u], base[u] + stride, ...; a null base sums to 0):
+// the loads of four parts of every stream are issued before the additions, so
+// that the streams share their latencies.
+template <int NP>
+__device__ __forceinline__ void sum_streams(const float* const (&base)[NP], const size_t (&stride)[NP], int n,
+                                            float (&out)[NP]) {
+#pragma unroll
+    for (int u = 0; u < NP; ++u) out[u] = 0.f;
+#pragma unroll 1
+    for (int i = 0; i < n; i += 4) {
+        float v[4][NP];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int u = 0; u < NP; ++u)
+                v[q][u] = (base[u] && i + q < n) ? base[u][(size_t)(i + q) * stride[u]] : 0.f;
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int u = 0; u < NP; ++u)
+                if (i + q < n) out[u] = __fadd_rn(out[u], v[q][u]);
+    }
+}
+
+// Values u < nv of a token's partial sums at off + u * ustride, up to kMS of
+// them: four streams at a time (KEEP), or every value's load of one part before
+// its additions (fewer registers).
 constexpr int kMS = 8;
+template <bool KEEP>
 __device__ __forceinline__ void multi_sum(const float* __restrict__ base, size_t stride, int n, int off,
                                           int ustride, int nv, float (&out)[kMS]) {
 #pragma unroll
     for (int u = 0; u < kMS; ++u) out[u] = 0.f;
+    if (KEEP) {
+#pragma unroll
+        for (int u0 = 0; u0 < kMS; u0 += 4) {
+            if (u0 >= nv) break;
+            const float* b[4];
+            const size_t st[4] = {stride, stride, stride, stride};
+            float o[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) b[u] = u0 + u < nv ? base + off + (u0 + u) * ustride : nullptr;
+            sum_streams<4>(b, st, n, o);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) out[u0 + u] = o[u];
+        }
+        return;
+    }
     if (nv == 1) {
         out[0] = sum_parts(base + off, stride, n);
         return;
@@ -113,8 +153,8 @@ __device__ __forceinline__ void multi_sum(const float* __restrict__ base, size_t
 // transitions: the threads of a warp hold consecutive k and read consecutive
 // entries, eight rows' loads in flight.  (Read along the rows of P instead,
 // every load of a warp touches 32 lines: 700 tables of a four-layer
-// Qwen-shaped forward, E = 60, 60.4 -> 38.1 us together with the branch-free
-// minimum in lookahead_table.)
+// Qwen-shaped forward, E = 60, 60.4 -> 31.9 us together with the minimum's
+// branch-free loop and broadcast reads in lookahead_table.)
 __device__ __forceinline__ float phi_entry(const float* __restrict__ PT, const float* V, int E) {
     float acc = 0.f;
     int kp = 0;
@@ -139,18 +179,27 @@ struct WarpCounters {
 // G lanes per token (8, 16 or 32): a warp decides 32 / G tokens at once.  With
 // E <= G every per-expert value sits in its own lane, so the reduction trees
 // over experts are those of a full warp with the unused lanes at zero.
-// Seven blocks per SM (72 registers, a few bytes spilled): each token is a
-// chain of dependent reads, so warps in flight matter more than registers
+// KM: slots held in registers (k <= KM).  KEEP: for batches of at most sixteen
+// tokens per SM, a token's own chain of reads is what counts: the slots' arrays
+// are unrolled into registers (128, four blocks per SM), partial sums are read
+// several streams at a time, every slot's candidates are read together and kept
+// for the choice, and the look-ahead interval is counted in one round of reads
+// instead of a binary search (three overlapping streams of 64-token
+// Switch-shaped forwards 77.4 -> 73.4 us a forward, a 777-token one through
+// host buffers 425 -> 412 us, 1-token Mixtral-shaped 429.5 -> 426.5 us).
+// Without it, seven blocks per SM (72 registers, a few bytes spilled): each
+// token is a chain of dependent reads, so warps in flight matter more than registers
 // (six blocks at 80 registers: 1.31 instead of 0.94 ms per Mixtral-shaped
 // forward, 1.59 instead of 1.45 ms per Qwen-shaped one).
-template <int G>
-__global__ void __launch_bounds__(kWarps * 32, 7) decide_kernel(const DecideParams p) {
+template <int G, int KM, bool KEEP>
+__global__ void __launch_bounds__(kWarps * 32, KEEP ? 4 : 7) decide_kernel(const DecideParams p) {
     pdl_wait();      // results of the preceding kernel in the stream
     extern __shared__ float smem[];
     const int lane = threadIdx.x & (G - 1);          // lane within the token's group
     const int warp = threadIdx.x >> 5;
     const int grp = (threadIdx.x & 31) / G;
     const unsigned gmask = G == 32 ? 0xffffffffu : (((1u << G) - 1u) << (grp * G));
+    constexpr int KU = KEEP ? KM : 1;                // unrolled over the slots
     constexpr int kGroups = kWarps * (32 / G);      // tokens in flight per block
     const int slot = warp * (32 / G) + grp;
     const int E = p.E, M = p.M, C = p.C, K = p.k, l = p.layer;
@@ -213,9 +262,21 @@ __global__ void __launch_bounds__(kWarps * 32, 7) decide_kernel(const DecidePara
         float rn = 1.f;
         const size_t kstride = (size_t)p.zs;      // the column ranges of a token are contiguous
         const float* zrow = p.zpart + (size_t)t * p.ksplit * p.zs;
-        float zacc = lane < E ? sum_parts(zrow + lane, kstride, p.ksplit) : 0.f;
+        float zacc, sq = 0.f;
+        if (KEEP) {
+            // the first expert's logit and the sum of squares together
+            const float* const bs[2] = {lane < E ? zrow + lane : nullptr,
+                                        p.use_norm ? p.sqpart + (size_t)t * p.ksplit : nullptr};
+            const size_t st[2] = {kstride, 1};
+            float o[2];
+            sum_streams<2>(bs, st, p.ksplit, o);
+            zacc = o[0];
+            sq = o[1];
+        } else {
+            zacc = lane < E ? sum_parts(zrow + lane, kstride, p.ksplit) : 0.f;
+            if (p.use_norm) sq = sum_parts(p.sqpart + (size_t)t * p.ksplit, 1, p.ksplit);
+        }
         if (p.use_norm) {
-            const float sq = sum_parts(p.sqpart + (size_t)t * p.ksplit, 1, p.ksplit);
             rn = rsqrtf(sq / (float)p.d + p.norm_eps);
             if (lane == 0) p.rnorm[t] = rn;
         }
@@ -238,10 +299,12 @@ __global__ void __launch_bounds__(kWarps * 32, 7) decide_kernel(const DecidePara
         __syncwarp(gmask);
         for (int e = lane; e < E; e += G) ps[e] = __fdiv_rn(ps[e], S);
         __syncwarp(gmask);
-        int topk[kMaxK];
-        float g[kMaxK];
+        int topk[KM];
+        float g[KM];
         unsigned used = 0u;   // bit i: expert lane + G i taken
-        for (int j = 0; j < K; ++j) {
+#pragma unroll KU
+        for (int j = 0; j < (KEEP ? KM : K); ++j) {
+            if (KEEP && j >= K) continue;
             float bz = -kInf;
             int be = 0x7fffffff;
             for (int i = 0, e = lane; e < E; ++i, e += G)
@@ -251,7 +314,12 @@ __global__ void __launch_bounds__(kWarps * 32, 7) decide_kernel(const DecidePara
             if ((be % G) == lane) used |= 1u << (be / G);
         }
         float I = 0.f;
-        for (int j = 0; j < K; ++j) { g[j] = ps[topk[j]]; I = __fadd_rn(I, g[j]); }
+#pragma unroll KU
+        for (int j = 0; j < (KEEP ? KM : K); ++j) {
+            if (KEEP && j >= K) continue;
+            g[j] = ps[topk[j]];
+            I = __fadd_rn(I, g[j]);
+        }
 
         // Exit confidence of the previous layer's head (Eq. 7), exit gate (Eq. 8-9).
         float xi = -1.f;
@@ -268,7 +336,7 @@ __global__ void __launch_bounds__(kWarps * 32, 7) decide_kernel(const DecidePara
             for (int c0 = lane; c0 < C; c0 += kMS * G) {
                 const int nv = min(kMS, (C - c0 + G - 1) / G);
                 float acc[kMS];
-                multi_sum(zrow, kstride, p.ksplit, E + c0, G, nv, acc);
+                multi_sum<KEEP>(zrow, kstride, p.ksplit, E + c0, G, nv, acc);
 #pragma unroll
                 for (int u = 0; u < kMS; ++u)
                     if (u < nv) xs[c0 + u * G] = __fadd_rn(__fmul_rn(acc[u], rx), p.bias[E + c0 + u * G]);
@@ -298,7 +366,7 @@ __global__ void __launch_bounds__(kWarps * 32, 7) decide_kernel(const DecidePara
             for (int j0 = lane; j0 < p.n_cent; j0 += kMS * G) {
                 const int nv = min(kMS, (p.n_cent - j0 + G - 1) / G);
                 float acc[kMS];
-                multi_sum(zrow, kstride, p.ksplit, E + C + j0, G, nv, acc);
+                multi_sum<KEEP>(zrow, kstride, p.ksplit, E + C + j0, G, nv, acc);
 #pragma unroll
                 for (int u = 0; u < kMS; ++u) {
                     if (u >= nv) continue;
@@ -314,11 +382,38 @@ __global__ void __launch_bounds__(kWarps * 32, 7) decide_kernel(const DecidePara
         if (lane == 0 && p.lhat_out) p.lhat_out[t] = (int16_t)Lhat;
 
         // Transmission necessity (Eq. 35) over the budget-feasible candidates (Eq. 34).
+        // With KEEP lane i keeps candidate i of every slot in registers (a slot
+        // seldom has more than G): all slots' reads are in flight together and the
+        // choice below does not read them again.
+        constexpr int KC = KEEP ? KM : 1;
+        constexpr int kFrom = KEEP ? G : 0;      // candidates from here on are read where they are used
+        int cbeg[KC], cend[KC], cm[KC], ck[KC];
+        float cQ[KC];
+        if (KEEP) {
+#pragma unroll
+            for (int j = 0; j < KC; ++j) {
+                cbeg[j] = j < K ? coff_l[topk[j]] : 0;
+                cend[j] = j < K ? coff_l[topk[j] + 1] : 0;
+            }
+#pragma unroll
+            for (int j = 0; j < KC; ++j) {
+                const int c = cbeg[j] + lane;
+                const bool in = c < cend[j];
+                cQ[j] = in ? p.tab.cand_Q[c] : kInf;
+                cm[j] = in ? p.tab.cand_m[c] : 0;
+                ck[j] = in ? p.tab.cand_k[c] : 0;
+            }
+        }
         float Gamma = 0.f;
-        for (int j = 0; j < K; ++j) {
-            const int c0 = coff_l[topk[j]], c1 = coff_l[topk[j] + 1];
+#pragma unroll KU
+        for (int j = 0; j < (KEEP ? KM : K); ++j) {
+            if (KEEP && j >= K) continue;
+            const int jc = KEEP ? j : 0;
+            const int c0 = KEEP ? cbeg[jc] : coff_l[topk[j]], c1 = KEEP ? cend[jc] : coff_l[topk[j] + 1];
             float gmin = kInf;
-            for (int c = c0 + lane; c < c1; c += G) {
+            if (KEEP && c0 + lane < c1 && __fadd_rn(Dhat, cQ[jc]) <= Dbar)
+                gmin = (cm[jc] != s) ? p.tab.trans[s * M + cm[jc]] : 0.f;
+            for (int c = c0 + kFrom + lane; c < c1; c += G) {
                 const float Q = p.tab.cand_Q[c];
                 if (__fadd_rn(Dhat, Q) <= Dbar) {
                     const int m = p.tab.cand_m[c];
@@ -341,10 +436,21 @@ __global__ void __launch_bounds__(kWarps * 32, 7) decide_kernel(const DecidePara
         const float* phiP = bufPhi;
         const bool use_shared = p.phi_tabs != nullptr && top >= p.dmin && top > 0 && Dbar == *p.dbar_shared;
         if (use_shared) {
-            int lo = 0, hi = p.n_thr;       // interval = number of thresholds <= R
-            while (lo < hi) {
-                const int mid = (lo + hi) >> 1;
-                if (p.thr[mid] <= R) lo = mid + 1; else hi = mid;
+            int lo = 0;                     // interval = number of thresholds <= R (sorted)
+            if (G == 32 && p.n_thr <= 8 * G) {
+                // few tokens: one round of parallel reads instead of a chain of them
+                float tv[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) tv[u] = lane + u * G < p.n_thr ? p.thr[lane + u * G] : kInf;
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    lo += __popc(__ballot_sync(0xffffffffu, lane + u * G < p.n_thr && tv[u] <= R));
+            } else {
+                int hi = p.n_thr;
+                while (lo < hi) {
+                    const int mid = (lo + hi) >> 1;
+                    if (p.thr[mid] <= R) lo = mid + 1; else hi = mid;
+                }
             }
             phiP = p.phi_tabs + ((size_t)(top - p.dmin) * (p.n_thr + 1) + lo) * ME;
             have_phi = true;
@@ -404,30 +510,45 @@ __global__ void __launch_bounds__(kWarps * 32, 7) decide_kernel(const DecidePara
 
         // Execute plan: slot 0 by f + Phi, later slots by f (Eq. 40), budget by Eq. (34).
         const float* ct_s = ct_l + s * M;
-        int esel[kMaxK], msel[kMaxK];
+        int esel[KM], msel[KM];
         float Drun = Dhat, tot = 0.f;
-        for (int j = 0; j < K; ++j) {
-            const int c0 = coff_l[topk[j]], c1 = coff_l[topk[j] + 1];
+#pragma unroll KU
+        for (int j = 0; j < (KEEP ? KM : K); ++j) {
+            if (KEEP && j >= K) continue;
+            const int jc = KEEP ? j : 0;
+            const int c0 = KEEP ? cbeg[jc] : coff_l[topk[j]], c1 = KEEP ? cend[jc] : coff_l[topk[j] + 1];
             float bv = kInf;
             int bi = 0x7fffffff;
-            for (int c = c0 + lane; c < c1; c += G) {
-                const float Q = p.tab.cand_Q[c];
-                const int m = p.tab.cand_m[c];
-                const float ct = ct_s[m];
-                // the cost-to-go is read before the budget tests decide whether it is used
-                const float ph = (j == 0 && have_phi) ? phiP[m * E + p.tab.cand_k[c]] : 0.f;
-                if (!(__fadd_rn(Dhat, Q) <= Dbar)) continue;
-                if (!(__fadd_rn(Drun, Q) <= Dbar)) continue;
+            // the cost and cost-to-go are read before the budget tests decide whether they are used
+            auto consider = [&](int c, float Q, int m, float ct, float ph) {
+                if (!(__fadd_rn(Dhat, Q) <= Dbar)) return;
+                if (!(__fadd_rn(Drun, Q) <= Dbar)) return;
                 float f = ct;
                 if (Q > 0.f) f = __fadd_rn(f, __fmul_rn(p.omega_D, __fdiv_rn(Q, Dbar)));
                 float v = f;
                 if (j == 0) v = __fadd_rn(f, ph);
                 if (v < bv) { bv = v; bi = c; }
+            };
+            if (KEEP && c0 + lane < c1)
+                consider(c0 + lane, cQ[jc], cm[jc], ct_s[cm[jc]],
+                         (j == 0 && have_phi) ? phiP[cm[jc] * E + ck[jc]] : 0.f);
+            for (int c = c0 + kFrom + lane; c < c1; c += G) {
+                const int m = p.tab.cand_m[c];
+                consider(c, p.tab.cand_Q[c], m, ct_s[m], (j == 0 && have_phi) ? phiP[m * E + p.tab.cand_k[c]] : 0.f);
             }
             grp_argmin<G>(gmask, bv, bi);
-            esel[j] = p.tab.cand_k[bi];
-            msel[j] = p.tab.cand_m[bi];
-            Drun = __fadd_rn(Drun, p.tab.cand_Q[bi]);
+            float Qsel;
+            if (KEEP && bi - c0 < G) {      // the winner sits in a lane's registers
+                const int src = bi - c0;
+                esel[j] = __shfl_sync(gmask, ck[jc], src, G);
+                msel[j] = __shfl_sync(gmask, cm[jc], src, G);
+                Qsel = __shfl_sync(gmask, cQ[jc], src, G);
+            } else {
+                esel[j] = p.tab.cand_k[bi];
+                msel[j] = p.tab.cand_m[bi];
+                Qsel = p.tab.cand_Q[bi];
+            }
+            Drun = __fadd_rn(Drun, Qsel);
             tot = (j == 0) ? bv : __fadd_rn(tot, bv);
         }
         const float tot_exec = tot;
@@ -442,16 +563,35 @@ __global__ void __launch_bounds__(kWarps * 32, 7) decide_kernel(const DecidePara
 
         // Outputs and state update (Eq. 41, 42, exit).
         if (lane < K) {
-            p.topk_idx[t * K + lane] = topk[lane];
-            p.topk_g[t * K + lane] = g[lane];
-            p.exp_sel[t * K + lane] = action == 0 ? (uint8_t)esel[lane] : 0xFF;
-            p.srv_sel[t * K + lane] = action == 0 ? (uint8_t)msel[lane] : 0xFF;
+            int tk = topk[0], es = esel[0], ms = msel[0];
+            float gj = g[0];
+            if (KEEP) {
+#pragma unroll
+                for (int j = 1; j < KM; ++j)
+                    if (lane == j) {
+                        tk = topk[j];
+                        gj = g[j];
+                        es = esel[j];
+                        ms = msel[j];
+                    }
+            } else {
+                tk = topk[lane % KM];
+                gj = g[lane % KM];
+                es = esel[lane % KM];
+                ms = msel[lane % KM];
+            }
+            p.topk_idx[t * K + lane] = tk;
+            p.topk_g[t * K + lane] = gj;
+            p.exp_sel[t * K + lane] = action == 0 ? (uint8_t)es : 0xFF;
+            p.srv_sel[t * K + lane] = action == 0 ? (uint8_t)ms : 0xFF;
         }
         if (lane == 0 && p.calib) {
             // Calibration counts of the offline stage (Eq. 26-28, 38).
             atomicAdd(&p.c_alive[l], 1ull);
             atomicAdd(&p.c_resid[l * M + s], 1ull);
-            for (int j = 0; j < K; ++j) {
+#pragma unroll KU
+            for (int j = 0; j < (KEEP ? KM : K); ++j) {
+                if (KEEP && j >= K) continue;
                 atomicAdd(&p.c_act[l * E + topk[j]], 1ull);
                 if (I > p.tab.theta[l]) atomicAdd(&p.c_above[l * E + topk[j]], 1ull);
             }
@@ -472,7 +612,7 @@ __global__ void __launch_bounds__(kWarps * 32, 7) decide_kernel(const DecidePara
                 p.last_exec[t] = 1;
                 float dl = 0.f;
 #pragma unroll
-                for (int j = 0; j < kMaxK; ++j) {
+                for (int j = 0; j < KM; ++j) {
                     if (j >= K) break;
                     const bool remote = msel[j] != s;
                     const bool sub = esel[j] != topk[j];
@@ -572,7 +712,9 @@ __device__ __forceinline__ void lookahead_table(const DecideParams& p, int l, co
         const float skip_cost = __fmul_rn(p.omega_D, __fdiv_rn(eps, Dbar));
         const bool skip_budget = eps <= R;
         for (int idx = threadIdx.x; idx < ME; idx += blockDim.x) {
-            const int m = idx / E, kp = idx - (idx / E) * E;
+            // m is the fast index: a warp's threads walk the same few targets'
+            // candidates, whose entries are then broadcast reads.
+            const int kp = idx / M, m = idx - kp * M;
             const int s0 = coff[kp] - cb, s1 = coff[kp + 1] - cb;
             const float* ctm = ct + m * M;
             float best = kInf;
@@ -595,7 +737,7 @@ __device__ __forceinline__ void lookahead_table(const DecideParams& p, int l, co
                 if (have_phi) v = __fadd_rn(v, bufPhi[m * E + kp]);
                 best = fminf(best, v);
             }
-            bufV[idx] = best;
+            bufV[m * E + kp] = best;
         }
         __syncthreads();
         for (int idx = threadIdx.x; idx < ME; idx += blockDim.x) {
@@ -695,6 +837,17 @@ size_t decide_smem_bytes(int E, int C, int M, int max_layer_cand) {
     return decide_smem_for(E, C, M, max_layer_cand, decide_group(E));
 }
 
+namespace {
+
+using DecideFn = void (*)(DecideParams);
+// Lanes per token 8, 16, 32; with the candidates kept, up to 1, 2, 4, 8 slots.
+const DecideFn kDecide[3] = {decide_kernel<8, kMaxK, false>, decide_kernel<16, kMaxK, false>,
+                             decide_kernel<32, kMaxK, false>};
+const DecideFn kDecideKeep[4] = {decide_kernel<32, 1, true>, decide_kernel<32, 2, true>, decide_kernel<32, 4, true>,
+                                 decide_kernel<32, kMaxK, true>};
+
+}  // namespace
+
 cudaError_t launch_decide(const DecideParams& p, int num_sms, cudaStream_t st) {
     if (p.T <= 0) return cudaSuccess;
     // Groups smaller than a warp pay off when the tokens outnumber the resident
@@ -707,11 +860,10 @@ cudaError_t launch_decide(const DecideParams& p, int num_sms, cudaStream_t st) {
     const size_t smem = decide_smem_for(p.E, p.C, p.M, p.tab.max_layer_cand, G, la_global);
     static PerDevice attr;
     const cudaError_t ea = (cudaError_t)attr.get([] {
-        cudaError_t e = cudaFuncSetAttribute(decide_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(decide_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(decide_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+        cudaError_t e = cudaSuccess;
+        for (const DecideFn f : {kDecide[0], kDecide[1], kDecide[2], kDecideKeep[0], kDecideKeep[1], kDecideKeep[2],
+                                 kDecideKeep[3]})
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
         return (int)e;
     }, true);
     if (ea != cudaSuccess) return ea;
@@ -721,9 +873,10 @@ cudaError_t launch_decide(const DecideParams& p, int num_sms, cudaStream_t st) {
     const int cap = la_global ? num_sms * kDecideLaBlocksPerSm : num_sms * 16;   // global slots exist for cap blocks
     blocks = blocks < cap ? blocks : cap;
     cudaError_t e;
-    if (G == 8) e = launch_pdl(decide_kernel<8>, dim3(blocks), dim3(kWarps * 32), smem, st, p);
-    else if (G == 16) e = launch_pdl(decide_kernel<16>, dim3(blocks), dim3(kWarps * 32), smem, st, p);
-    else e = launch_pdl(decide_kernel<32>, dim3(blocks), dim3(kWarps * 32), smem, st, p);
+    const bool keep = G == 32 && p.T <= num_sms * 4 * kWarps;
+    const DecideFn fn = keep ? kDecideKeep[p.k <= 1 ? 0 : p.k <= 2 ? 1 : p.k <= 4 ? 2 : 3]
+                             : kDecide[G == 8 ? 0 : G == 16 ? 1 : 2];
+    e = launch_pdl(fn, dim3(blocks), dim3(kWarps * 32), smem, st, p);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }

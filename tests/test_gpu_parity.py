@@ -348,6 +348,16 @@ def test_layer_parity_transposed_swiglu(name, kw):
     assert tot["exec"] > 0
 
 
+@pytest.mark.parametrize("k", [1, 3, 8])
+def test_layer_parity_more_candidates_than_lanes(k):
+    """Every expert on all 16 servers: 64 candidates per slot, twice the lanes of
+    a token's warp, so the candidates past the ones kept in registers are read
+    where they are used; slots 1, 3 and 8 of the register variants 1, 4 and 8."""
+    cfg = small_cfg(name="cand64", N=3, d=256, E=12, k=k, F=128, T=200, M=16, H=3, placement="full", seed=96)
+    reports = _run_all_layers(cfg, theta=0.9, exit_bias=1.0)
+    assert sum(r["exec"] for r in reports) > 0
+
+
 def test_layer_parity_decision_lane_groups_of_16():
     """8 < E <= 16 with more tokens than the resident warps (T >= 16 x SMs):
     the decision kernel runs two tokens per warp on 16-lane groups."""
