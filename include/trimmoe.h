@@ -244,7 +244,8 @@ typedef struct {
     uint64_t launches;            /* kernels launched by the library */
     uint64_t layer_calls;         /* layers processed */
     double gemm_flops;            /* 2*M*N*K of the grouped FFN GEMMs that ran */
-    /* Device time per kernel family in ms (profile != 0 only). */
+    /* Device time per kernel family in ms (profile != 0 only).  Up to 1024 tokens
+     * compaction and gather are one launch, counted in ms_compact. */
     double ms_decide, ms_compact, ms_gather, ms_gemm_up, ms_gemm_down, ms_combine;
     uint64_t n_gemm_up, n_gemm_down;
     double flops_gemm_up, flops_gemm_down;

@@ -11,6 +11,7 @@
 // scatter in which each chunk's block derives its base and the group offsets
 // from all chunks' counts and each of its warps walks its 32 tokens in order,
 // ranking equal buckets with __match_any_sync (one pass for a single chunk).
+#include <algorithm>
 #include <mutex>
 #include <string>
 
@@ -21,6 +22,7 @@ namespace tmoe {
 namespace {
 
 constexpr int kChunk = 256;
+constexpr int kFusedMaxT = 1024;     // compaction and gather in one launch
 
 __global__ void __launch_bounds__(kChunk) count_kernel(const CompactParams p) {
     pdl_wait();      // results of the preceding kernel in the stream
@@ -191,66 +193,208 @@ __global__ void __launch_bounds__(kChunk) scatter_kernel(const CompactParams p) 
     }
 }
 
-// Xp[row] = expert input of the row's token: bf16(h * r * gamma) with the
-// pre-FFN RMSNorm, or h itself without it; one warp per row, gamma staged in
-// shared memory once per block, kGU chunks of 16 bytes per lane in flight.
+// Expert input of token t, chunks [cbeg, cend) of 16 bytes, by one warp:
+// bf16(h * r * gamma) with the pre-FFN RMSNorm (gamma staged in sg), or h itself
+// without it; kGU chunks per lane in flight.
 constexpr int kGU = 8;
 constexpr int kMaxGatherD = 16384;   // gamma staged in shared memory (32 KB)
+__device__ __forceinline__ void gather_chunks(const uint4* __restrict__ src, uint4* __restrict__ dst, int cbeg, int cend,
+                                              int lane, bool norm, float rn, const uint4* sg) {
+    for (int c0 = cbeg + lane; c0 < cend; c0 += 32 * kGU) {
+        uint4 hv[kGU];
+#pragma unroll
+        for (int u = 0; u < kGU; ++u)
+            if (c0 + 32 * u < cend) hv[u] = src[c0 + 32 * u];
+#pragma unroll
+        for (int u = 0; u < kGU; ++u) {
+            const int c = c0 + 32 * u;
+            if (c >= cend) continue;
+            if (!norm) {
+                dst[c] = hv[u];
+                continue;
+            }
+            const uint4 gv = sg[c];
+            uint4 o;
+            o.x = pack_bf16x2(bf16_lo(hv[u].x) * rn * bf16_lo(gv.x), bf16_hi(hv[u].x) * rn * bf16_hi(gv.x));
+            o.y = pack_bf16x2(bf16_lo(hv[u].y) * rn * bf16_lo(gv.y), bf16_hi(hv[u].y) * rn * bf16_hi(gv.y));
+            o.z = pack_bf16x2(bf16_lo(hv[u].z) * rn * bf16_lo(gv.z), bf16_hi(hv[u].z) * rn * bf16_hi(gv.z));
+            o.w = pack_bf16x2(bf16_lo(hv[u].w) * rn * bf16_lo(gv.w), bf16_hi(hv[u].w) * rn * bf16_hi(gv.w));
+            dst[c] = o;
+        }
+    }
+}
 
+// Xp[row] of every compacted row, one warp per row or row segment, gamma staged
+// in shared memory once per block.
 __global__ void __launch_bounds__(256) gather_kernel(const int32_t* __restrict__ perm,
-                                                     const int32_t* __restrict__ goff, int E, int k,
-                                                     int d, const __nv_bfloat16* __restrict__ h,
-                                                     const float* __restrict__ rnorm,
-                                                     const __nv_bfloat16* __restrict__ gamma,
-                                                     __nv_bfloat16* __restrict__ Xp, int nseg) {
+                                                     const int32_t* __restrict__ goff, const GatherParams p) {
     pdl_wait();      // results of the preceding kernel in the stream
     pdl_trigger();   // single-wave grid: let the next kernel be scheduled now
     extern __shared__ uint4 sg[];      // gamma, d / 8 chunks
-    const int nrows = goff[E + 1];
-    const int routed = goff[E];
+    const int nrows = goff[p.E + 1];
+    const int routed = goff[p.E];
     const int lane = threadIdx.x & 31;
-    const int nchunk = d >> 3;
-    if (gamma) {
-        const uint4* gv4 = reinterpret_cast<const uint4*>(gamma);
+    const int nchunk = p.d >> 3;
+    if (p.gamma) {
+        const uint4* gv4 = reinterpret_cast<const uint4*>(p.gamma);
         for (int c = threadIdx.x; c < nchunk; c += blockDim.x) sg[c] = __ldg(gv4 + c);
         __syncthreads();
     }
-    // A warp copies one of nseg segments of a row (nseg > 1 for decode-sized
-    // batches, so that a row's loads are in flight together).
-    const int seg_chunks = (nchunk + nseg - 1) / nseg;
-    const long long nunits = (long long)nrows * nseg;
-    for (long long unit = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; unit < nunits;
-         unit += (gridDim.x * blockDim.x) >> 5) {
-        const int r = (int)(unit / nseg);
-        const int cbeg = (int)(unit - (long long)r * nseg) * seg_chunks;
-        const int cend = min(nchunk, cbeg + seg_chunks);
+    for (int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < nrows; r += (gridDim.x * blockDim.x) >> 5) {
         const int code = perm[r];
-        const int t = r < routed ? code / k : code;
-        const uint4* __restrict__ src = reinterpret_cast<const uint4*>(h + (size_t)t * d);
-        uint4* __restrict__ dst = reinterpret_cast<uint4*>(Xp + (size_t)r * d);
-        const float rn = gamma ? rnorm[t] : 1.f;
-        for (int c0 = cbeg + lane; c0 < cend; c0 += 32 * kGU) {
-            uint4 hv[kGU];
+        const int t = r < routed ? code / p.k : code;
+        gather_chunks(reinterpret_cast<const uint4*>(p.h + (size_t)t * p.d),
+                      reinterpret_cast<uint4*>(p.Xp + (size_t)r * p.d), 0, nchunk, lane, p.gamma != nullptr,
+                      p.gamma ? p.rnorm[t] : 1.f, sg);
+    }
+}
+
+// Small batches (T <= 32 NW): compaction and gather in one launch.  At these
+// sizes either is a few dependent reads long, so what a launch less saves is
+// most of what they cost (64-token Switch-shaped
+// forwards 73.4 -> 72.6 us, a 777-token one through host buffers 413 -> 405 us,
+// a 333-token Qwen-shaped one alone 1020 -> 995 us).  Every block
+// ranks all pairs itself (a token's action and experts are 1 + k bytes), keeps
+// the rows of its own range of the output order and gathers those; block 0 also
+// writes the group offsets and the counters.  A warp takes one of nseg segments
+// of a row, so that a row's loads are in flight together.
+constexpr int kFusedRows = 64;       // rows of one block at most
+template <int NW>
+__global__ void __launch_bounds__(NW * 32) compact_gather_kernel(const CompactParams p, const GatherParams q, int nseg) {
+    extern __shared__ uint4 sg[];      // gamma, d / 8 chunks
+    __shared__ int run[NW][kMaxE + 1];
+    __shared__ int goff_s[kMaxE + 2], total[kMaxE + 1], mine[kFusedRows];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int nb = p.E + 1;
+    const int nchunk = q.d >> 3;
+    // gamma is a weight: staged before the programmatic wait
+    if (q.gamma) {
+        const uint4* gv4 = reinterpret_cast<const uint4*>(q.gamma);
+        for (int c = threadIdx.x; c < nchunk; c += blockDim.x) sg[c] = __ldg(gv4 + c);
+    }
+    for (int i = threadIdx.x; i < NW * nb; i += blockDim.x) run[i / nb][i % nb] = 0;
+    __syncthreads();
+    pdl_wait();      // results of the preceding kernel in the stream
+    pdl_trigger();   // single-wave grid: let the next kernel be scheduled now
+
+    const int t0 = warp * 32;
+    const int tn = max(0, min(32, p.T - t0));
+    const unsigned lt_mask = (1u << lane) - 1u;
+    const int npairs = tn * p.k;
+    const int act = lane < tn ? p.action[t0 + lane] : 3;
+    const bool take = p.has_shared && act <= 1;
+    // Pass 1: this warp's count per bucket.
+    for (int q0 = 0; q0 < npairs; q0 += 32) {
+        const int i = q0 + lane;
+        const int tl = i / p.k;                                    // token of this pair within the warp
+        const int a = __shfl_sync(0xffffffffu, act, tl & 31);
+        int key = -1;
+        if (i < npairs && a == 0) key = p.exp_sel[t0 * p.k + i];
+        const unsigned peers = __match_any_sync(0xffffffffu, key);
+        if (key >= 0 && (peers & lt_mask) == 0) run[warp][key] += __popc(peers);
+        __syncwarp();
+    }
+    const unsigned ball = __ballot_sync(0xffffffffu, take);
+    if (lane == 0) run[warp][p.E] = __popc(ball);
+    __syncthreads();
+    // Starting positions: per bucket over the warps, then over the buckets.
+    for (int e = threadIdx.x; e < nb; e += blockDim.x) {
+        int acc = 0;
+#pragma unroll 8
+        for (int w = 0; w < NW; ++w) {
+            const int c = run[w][e];
+            run[w][e] = acc;
+            acc += c;
+        }
+        total[e] = acc;
+    }
+    __syncthreads();
+    if (warp == 0) {
+        int base = 0;
+        unsigned long long touched = 0;
+        for (int e0 = 0; e0 < nb; e0 += 32) {
+            const int e = e0 + lane;
+            const int c = e < nb ? total[e] : 0;
+            int incl = c;
 #pragma unroll
-            for (int u = 0; u < kGU; ++u)
-                if (c0 + 32 * u < cend) hv[u] = src[c0 + 32 * u];
-#pragma unroll
-            for (int u = 0; u < kGU; ++u) {
-                const int c = c0 + 32 * u;
-                if (c >= cend) continue;
-                if (!gamma) {
-                    dst[c] = hv[u];
-                    continue;
-                }
-                const uint4 gv = sg[c];
-                uint4 o;
-                o.x = pack_bf16x2(bf16_lo(hv[u].x) * rn * bf16_lo(gv.x), bf16_hi(hv[u].x) * rn * bf16_hi(gv.x));
-                o.y = pack_bf16x2(bf16_lo(hv[u].y) * rn * bf16_lo(gv.y), bf16_hi(hv[u].y) * rn * bf16_hi(gv.y));
-                o.z = pack_bf16x2(bf16_lo(hv[u].z) * rn * bf16_lo(gv.z), bf16_hi(hv[u].z) * rn * bf16_hi(gv.z));
-                o.w = pack_bf16x2(bf16_lo(hv[u].w) * rn * bf16_lo(gv.w), bf16_hi(hv[u].w) * rn * bf16_hi(gv.w));
-                dst[c] = o;
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += v;
+            }
+            if (e < nb) goff_s[e] = base + incl - c;
+            touched += __popc(__ballot_sync(0xffffffffu, e < p.E && c > 0));
+            base += __shfl_sync(0xffffffffu, incl, 31);
+        }
+        if (lane == 0) goff_s[nb] = base;
+        if (blockIdx.x == 0) {
+            __syncwarp();
+            for (int e = lane; e <= nb; e += 32) p.goff[e] = goff_s[e];
+            if (lane == 0) {
+                atomicAdd(&p.ctr->pairs_total, (unsigned long long)(base - total[p.E]));
+                atomicAdd(&p.ctr->shared_rows, (unsigned long long)total[p.E]);
+                atomicAdd(&p.ctr->experts_touched, touched);
+                if (total[p.E] > 0) atomicAdd(&p.ctr->shared_touched, 1ull);
             }
         }
+    }
+    __syncthreads();
+    // This block's units (row, segment) and the rows they touch.
+    const int nrows = goff_s[nb], routed = goff_s[p.E];
+    const int per = (nrows * nseg + (int)gridDim.x - 1) / (int)gridDim.x;
+    const int u0 = min(nrows * nseg, (int)blockIdx.x * per), u1 = min(nrows * nseg, u0 + per);
+    const int r0 = u0 / nseg, r1 = (u1 + nseg - 1) / nseg;
+    // A row's entries are written by the block of its first unit.
+    const int w0 = (u0 + nseg - 1) / nseg;
+    // Pass 2: positions; each block keeps its own rows.
+    for (int q0 = 0; q0 < npairs; q0 += 32) {
+        const int i = q0 + lane;
+        const int tl = i / p.k;
+        const int a = __shfl_sync(0xffffffffu, act, tl & 31);
+        const int code = t0 * p.k + i;
+        int key = -1;
+        if (i < npairs) {
+            if (a == 0) key = p.exp_sel[code];
+            else if (blockIdx.x == 0) p.pos_pair[code] = -1;
+        }
+        const unsigned peers = __match_any_sync(0xffffffffu, key);
+        if (key >= 0) {
+            const int pos = goff_s[key] + run[warp][key] + __popc(peers & lt_mask);
+            if (pos >= r0 && pos < r1) {
+                mine[pos - r0] = code;
+                if (pos >= w0) {
+                    p.perm[pos] = code;
+                    p.pos_pair[code] = pos;
+                }
+            }
+        }
+        __syncwarp();
+        if (key >= 0 && (peers & lt_mask) == 0) run[warp][key] += __popc(peers);
+        __syncwarp();
+    }
+    if (p.has_shared && lane < tn) {
+        if (take) {
+            const int pos = routed + run[warp][p.E] + __popc(ball & lt_mask);
+            if (pos >= r0 && pos < r1) {
+                mine[pos - r0] = t0 + lane;
+                if (pos >= w0) {
+                    p.perm[pos] = t0 + lane;
+                    p.pos_sh[t0 + lane] = pos - routed;
+                }
+            }
+        } else if (blockIdx.x == 0) {
+            p.pos_sh[t0 + lane] = -1;
+        }
+    }
+    __syncthreads();
+    const int seg_chunks = (nchunk + nseg - 1) / nseg;
+    for (int u = u0 + warp; u < u1; u += NW) {
+        const int r = u / nseg;
+        const int cbeg = (u - r * nseg) * seg_chunks;
+        const int code = mine[r - r0];
+        const int t = r < routed ? code / p.k : code;
+        gather_chunks(reinterpret_cast<const uint4*>(q.h + (size_t)t * q.d),
+                      reinterpret_cast<uint4*>(q.Xp + (size_t)r * q.d), cbeg, min(nchunk, cbeg + seg_chunks), lane,
+                      q.gamma != nullptr, q.gamma ? q.rnorm[t] : 1.f, sg);
     }
 }
 
@@ -269,12 +413,11 @@ cudaError_t launch_compact(const CompactParams& p, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_gather(const int32_t* perm, const int32_t* goff, int E, int k, int d,
-                          const __nv_bfloat16* h, const float* rnorm, const __nv_bfloat16* gamma,
-                          __nv_bfloat16* Xp, int max_rows, int num_sms, cudaStream_t st) {
+cudaError_t launch_gather(const int32_t* perm, const int32_t* goff, const GatherParams& q, int max_rows, int num_sms,
+                          cudaStream_t st) {
     if (max_rows <= 0) return cudaSuccess;
-    if (d > kMaxGatherD) return cudaErrorInvalidValue;
-    const size_t smem = gamma ? (size_t)d * 2 : 0;
+    if (q.d > kMaxGatherD) return cudaErrorInvalidValue;
+    const size_t smem = q.gamma ? (size_t)q.d * 2 : 0;
     static PerDevice occ;
     const int per_sm = occ.get([] {
         int n = 0;
@@ -283,13 +426,41 @@ cudaError_t launch_gather(const int32_t* perm, const int32_t* goff, int E, int k
             n = 1;
         return n;
     });
-    // Decode-sized batches: one row segment (a step of kGU chunks per lane) per warp.
-    const int steps = ((d >> 3) + 32 * kGU - 1) / (32 * kGU);
-    const int nseg = max_rows <= 512 && steps > 1 ? steps : 1;
-    long long want = ((long long)max_rows * nseg + 7) / 8;
+    const long long want = ((long long)max_rows + 7) / 8;
     const int blocks = (int)(want < (long long)num_sms * per_sm ? want : (long long)num_sms * per_sm);
-    const cudaError_t e = launch_pdl(gather_kernel, dim3(blocks), dim3(256), smem, st, perm, goff, E, k, d, h, rnorm,
-                                     gamma, Xp, nseg);
+    const cudaError_t e = launch_pdl(gather_kernel, dim3(blocks), dim3(256), smem, st, perm, goff, q);
+    if (e != cudaSuccess) return e;
+    return cudaGetLastError();
+}
+
+bool compact_gather_fits(int T) { return T <= kFusedMaxT; }
+
+cudaError_t launch_compact_gather(const CompactParams& p, const GatherParams& q, int num_sms, cudaStream_t st) {
+    if (p.T <= 0) return cudaSuccess;
+    if (q.d > kMaxGatherD || p.T > kFusedMaxT) return cudaErrorInvalidValue;
+    const size_t smem = q.gamma ? (size_t)q.d * 2 : 0;
+    const int max_rows = p.T * p.k + (p.has_shared ? p.T : 0);
+    static PerDevice attr;               // gamma beside the static arrays can pass 48 KB
+    const cudaError_t ea = (cudaError_t)attr.get([] {
+        cudaError_t e = cudaFuncSetAttribute(compact_gather_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             kMaxGatherD * 2);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(compact_gather_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     kMaxGatherD * 2);
+        return (int)e;
+    }, true);
+    if (ea != cudaSuccess) return ea;
+    // A row segment is a step of kGU chunks per lane; the grid is one wave (one
+    // block of 1024 threads per SM, or two of 256), and no block gets more rows
+    // than it has places for (at most ceil(9 * 1024 / 62) = 149 blocks).
+    const int steps = ((q.d >> 3) + 32 * kGU - 1) / (32 * kGU);
+    const int nseg = max_rows <= 512 ? steps : 1;
+    const int nw = p.T <= 256 ? 8 : 32;
+    const int want = (max_rows * nseg + nw - 1) / nw;
+    const int least = (max_rows + kFusedRows - 3) / (kFusedRows - 2);      // a range touches at most two rows in part
+    const int blocks = std::max(least, std::min(want, nw == 8 ? 2 * num_sms : num_sms));
+    const cudaError_t e = p.T <= 256 ? launch_pdl(compact_gather_kernel<8>, dim3(blocks), dim3(256), smem, st, p, q, nseg)
+                                     : launch_pdl(compact_gather_kernel<32>, dim3(blocks), dim3(1024), smem, st, p, q, nseg);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }

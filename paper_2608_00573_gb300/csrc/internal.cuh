@@ -157,6 +157,16 @@ struct CompactParams {
     DevCounters* ctr;
 };
 
+// The expert inputs' gather (see gather_chunks): row r of Xp from the token of
+// compacted row r; gamma null: the hidden state itself.
+struct GatherParams {
+    int E, k, d;
+    const __nv_bfloat16* h;
+    const float* rnorm;
+    const __nv_bfloat16* gamma;
+    __nv_bfloat16* Xp;
+};
+
 struct GemmLaunch {
     const CUtensorMap* tmA;
     const CUtensorMap* tmB;
@@ -271,9 +281,11 @@ struct LaLayer {
 cudaError_t launch_lookahead_all(const DecideParams& p, const LaLayer* layers, int n_layers, int max_thr,
                                  int max_depth, cudaStream_t st);
 cudaError_t launch_compact(const CompactParams& p, cudaStream_t st);
-cudaError_t launch_gather(const int32_t* perm, const int32_t* goff, int E, int k, int d,
-                          const __nv_bfloat16* h, const float* rnorm, const __nv_bfloat16* gamma,
-                          __nv_bfloat16* Xp, int max_rows, int num_sms, cudaStream_t st);
+cudaError_t launch_gather(const int32_t* perm, const int32_t* goff, const GatherParams& q, int max_rows, int num_sms,
+                          cudaStream_t st);
+// Both in one launch, for batches of up to compact_gather_fits tokens.
+bool compact_gather_fits(int T);
+cudaError_t launch_compact_gather(const CompactParams& p, const GatherParams& q, int num_sms, cudaStream_t st);
 cudaError_t launch_grouped_gemm(const GemmLaunch& g, int num_sms, cudaStream_t st);
 cudaError_t launch_splitk_finish(const GemmLaunch& g, int num_sms, cudaStream_t st);
 int grouped_gemm_ksplit(int est_tiles, int nkb, int num_sms);

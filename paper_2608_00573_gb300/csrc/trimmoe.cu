@@ -1112,13 +1112,17 @@ static trimmoe_status layer_step_impl(trimmoe_handle h, int layer, int T, trimmo
     cp.pos_pair = h->pos_pair;
     cp.pos_sh = h->pos_sh;
     cp.ctr = h->ctr;
-    e = h->timed(K_COMPACT, st, [&] { return launch_compact(cp, st); });
-    if (e != cudaSuccess) return h->fail(TRIMMOE_ERR_CUDA, std::string("compact: ") + cudaGetErrorString(e));
+    const GatherParams gp{E, K, d, hid, h->rnorm, gamma, h->Xp};
+    const bool fused = compact_gather_fits(T);      // counted as compaction
     const int max_rows = T * K + (has_sh ? T : 0);
-    e = h->timed(K_GATHER, st, [&] {
-        return launch_gather(h->perm, h->goff, E, K, d, hid, h->rnorm, gamma, h->Xp, max_rows, h->num_sms, st);
+    e = h->timed(K_COMPACT, st, [&] {
+        return fused ? launch_compact_gather(cp, gp, h->num_sms, st) : launch_compact(cp, st);
     });
-    if (e != cudaSuccess) return h->fail(TRIMMOE_ERR_CUDA, std::string("gather: ") + cudaGetErrorString(e));
+    if (e != cudaSuccess) return h->fail(TRIMMOE_ERR_CUDA, std::string("compact: ") + cudaGetErrorString(e));
+    if (!fused) {
+        e = h->timed(K_GATHER, st, [&] { return launch_gather(h->perm, h->goff, gp, max_rows, h->num_sms, st); });
+        if (e != cudaSuccess) return h->fail(TRIMMOE_ERR_CUDA, std::string("gather: ") + cudaGetErrorString(e));
+    }
 
     GemmLaunch g1{};
     g1.tmA = &h->tmXp;
@@ -1186,9 +1190,9 @@ static trimmoe_status layer_step_impl(trimmoe_handle h, int layer, int T, trimmo
     if (e != cudaSuccess) return h->fail(TRIMMOE_ERR_CUDA, std::string("gemm down: ") + cudaGetErrorString(e));
     h->n_gemm_up++;
     h->n_gemm_down++;
-    // router, decide, count (more than 256 tokens), scatter, gather, gate/up GEMM, down GEMM
+    // router, decide, compaction (count, scatter, gather, or one), gate/up GEMM, down GEMM
     // (+ look-ahead tables, split-K finishes)
-    h->launches += (T > 256 ? 7 : 6) + (tabs_here ? 1 : 0) + (g1.ksplit > 1 ? 1 : 0) + (g2.ksplit > 1 ? 1 : 0);
+    h->launches += (fused ? 5 : 7) + (tabs_here ? 1 : 0) + (g1.ksplit > 1 ? 1 : 0) + (g2.ksplit > 1 ? 1 : 0);
     if (has_sh) {
         GemmLaunch s1 = g1;
         s1.ksplit = 1;

@@ -348,6 +348,16 @@ def test_layer_parity_transposed_swiglu(name, kw):
     assert tot["exec"] > 0
 
 
+@pytest.mark.parametrize("T,kw", [(1, {}), (31, {}), (256, {}), (257, {}), (1024, dict(E=128, k=8)), (1025, {})])
+def test_layer_parity_compaction_sizes(T, kw):
+    """Compaction and gather in one launch up to 1024 tokens (8 warps per block to
+    256, 32 above, at most 64 rows per block: 9216 rows at 1024 tokens with eight
+    slots and a shared expert), in three launches above."""
+    cfg = small_cfg(name="fuse", **{**dict(N=2, d=256, E=20, k=3, F=128, F_sh=128, M=8, H=2, seed=95), **kw}, T=T)
+    reports = _run_all_layers(cfg, theta=0.7, exit_bias=1.0, row_sample=np.arange(0, T, 1 + T // 200))
+    assert T == 1 or sum(r["exec"] for r in reports) > 0
+
+
 @pytest.mark.parametrize("k", [1, 3, 8])
 def test_layer_parity_more_candidates_than_lanes(k):
     """Every expert on all 16 servers: 64 candidates per slot, twice the lanes of
