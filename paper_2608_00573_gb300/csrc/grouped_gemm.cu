@@ -29,6 +29,10 @@
 // Every mbarrier wait is bounded (2 s); on expiry the kernel records an error
 // word, stops issuing work, frees its TMEM and returns.
 //
+// Small-batch variant (few rows per group: the weights' stream bounds the
+// launch): 128 x 128 tiles, two CTAs per SM, the K range split for the smallest
+// batches; described at the kernel.
+//
 // Pair variant (launches whose groups are large): clusters of two CTAs on two
 // SMs issue tcgen05.mma.cta_group::2 with M = 256, N = 256.  Each CTA stages
 // its own 128 rows of A and its own half (128 output columns) of B, 32 KB per
@@ -82,6 +86,7 @@ struct __align__(8) SmemTail {
     uint32_t tmem_base;
     int abort_flag;
     int total_tiles;
+    int a_rows;                    // small-batch kernel: activation rows staged
     int tile_start[kMaxGroups + 1];
     int gstart[kMaxGroups];
     int gcnt[kMaxGroups];
@@ -99,10 +104,11 @@ struct Tile {
 // Per-group tile counts from the device-side group offsets (tile_rows rows per
 // row tile); one warp: 32 groups' offsets loaded at once, tile counts
 // prefix-summed with shuffles (integer sums, the same table as a serial loop).
+// Returns the largest group's rows in every lane.
 template <class Tail>
-__device__ __forceinline__ void build_tile_table(Tail* tl, const int* goff, int first_group, int ngroups,
+__device__ __forceinline__ int build_tile_table(Tail* tl, const int* goff, int first_group, int ngroups,
                                                  int n_tiles_n, int tile_rows, int lane) {
-    int carry = 0;
+    int carry = 0, most = 0;
     for (int g0 = 0; g0 < ngroups; g0 += 32) {
         const int g = g0 + lane;
         int st = 0, cnt = 0, nt = 0;
@@ -123,12 +129,16 @@ __device__ __forceinline__ void build_tile_table(Tail* tl, const int* goff, int 
             tl->tile_start[g] = carry + incl - nt;
         }
         carry += __shfl_sync(0xffffffffu, incl, 31);
+        most = max(most, cnt);
     }
     if (lane == 0) {
         tl->tile_start[ngroups] = carry;
         tl->total_tiles = carry;
         tl->abort_flag = 0;
     }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) most = max(most, __shfl_xor_sync(0xffffffffu, most, o));
+    return most;
 }
 
 // Tile t -> (group, row tile, column tile).  Within a group the row tiles are
@@ -195,32 +205,14 @@ __device__ __forceinline__ void store_row32(__nv_bfloat16* dst, const float (&v)
 }
 
 // Epilogue of one tile for one warp: TMEM lane quarter q (rows q*32 + lane),
-// all BN accumulator columns at tb; K range kr when the K dimension is split.
-__device__ __forceinline__ void epilogue_tile(uint32_t tb, int row, const Tile& ti, int kr, int ksplit,
-                                              int epi_mode, __nv_bfloat16* __restrict__ out, int ldo,
+// all BN accumulator columns at tb.
+__device__ __forceinline__ void epilogue_tile(uint32_t tb, int row, const Tile& ti, int epi_mode,
+                                              __nv_bfloat16* __restrict__ out, int ldo,
                                               const __nv_bfloat16* __restrict__ res, int ldr,
-                                              const RopeEpi& rp, float* __restrict__ partial, int ldp,
-                                              size_t pstride) {
+                                              const RopeEpi& rp) {
     const bool valid = row < ti.rows;
     __nv_bfloat16* orow = out + (size_t)(ti.out_row + (valid ? row : 0)) * ldo;
-    if (ksplit > 1) {
-        // fp32 partial sums of this K range; the finish kernel adds the ranges.
-        float* prow = partial + (size_t)kr * pstride + (size_t)(ti.out_row + (valid ? row : 0)) * ldp +
-                      ti.nt * BN;
-#pragma unroll 1
-        for (int c = 0; c < BN; c += 32) {
-            uint32_t r[32];
-            tmem_ld_32x32(tb + c, r);
-            tmem_ld_wait();
-            if (valid) {
-                float4* d4 = reinterpret_cast<float4*>(prow + c);
-#pragma unroll
-                for (int q4 = 0; q4 < 8; ++q4)
-                    d4[q4] = make_float4(__uint_as_float(r[4 * q4]), __uint_as_float(r[4 * q4 + 1]),
-                                         __uint_as_float(r[4 * q4 + 2]), __uint_as_float(r[4 * q4 + 3]));
-            }
-        }
-    } else if (epi_mode == EPI_SWIGLU) {
+    if (epi_mode == EPI_SWIGLU) {
 #pragma unroll 1
         for (int c = 0; c < BN / 2; c += 32) {
             uint32_t gr[32], ur[32];
@@ -341,8 +333,7 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                     int out_rebase, int K, int n_tiles_n, int b_rows_per_group, int epi_mode,
                     __nv_bfloat16* __restrict__ out, int ldo, int* err,
                     const __nv_bfloat16* __restrict__ res, int ldr, const RopeEpi rp,
-                    int mblk, int ksplit, float* __restrict__ partial,
-                    int ldp, size_t pstride) {
+                    int mblk) {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw_addr = smem_u32(smem_raw);
     const uint32_t pad = ((raw_addr + 1023u) & ~1023u) - raw_addr;
@@ -381,8 +372,7 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     if (warp == 0) build_tile_table(tl, goff, first_group, ngroups, n_tiles_n, BM, lane);
     __syncthreads();
     const int ntiles = tl->total_tiles;
-    const int total = ntiles * ksplit;    // unit u: tile u % ntiles, K range u / ntiles
-    if ((int)blockIdx.x >= total) {
+    if ((int)blockIdx.x >= ntiles) {
         if (warp == 0) {
             __syncwarp();
             tc_fence_after();
@@ -392,18 +382,16 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     }
     const int base0 = tl->gstart[0];
     const int nkb = K / BK;
-    const int kbr = nkb / ksplit;         // k blocks per range
     volatile int* abort_flag = &tl->abort_flag;
 
     if (warp == 0) {
         if (lane == 0) {
             // ---------------------------------------------------- producer
             int it = 0;
-            for (int t = blockIdx.x; t < total && !*abort_flag; t += gridDim.x) {
-                const Tile ti = map_tile(tl, t % ntiles, ngroups, n_tiles_n, base0, a_rebase, out_rebase,
+            for (int t = blockIdx.x; t < ntiles && !*abort_flag; t += gridDim.x) {
+                const Tile ti = map_tile(tl, t, ngroups, n_tiles_n, base0, a_rebase, out_rebase,
                                          b_rows_per_group, mblk, BM, 0, 0);
-                const int kb0 = (t / ntiles) * kbr;
-                for (int kb = kb0; kb < kb0 + kbr; ++kb, ++it) {
+                for (int kb = 0; kb < nkb; ++kb, ++it) {
                     const int s = it % STAGES;
                     const uint32_t ph = (it / STAGES) & 1;
                     if (!mbar_wait_bounded(smem_u32(&tl->empty[s]), ph ^ 1, abort_flag, err,
@@ -431,7 +419,7 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             constexpr uint32_t idesc = idesc_bf16_f32(BM, BN);
             int it = 0, tl_i = 0;
             bool ok = true;
-            for (int t = blockIdx.x; t < total && ok; t += gridDim.x, ++tl_i) {
+            for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++tl_i) {
                 const int buf = tl_i & 1;
                 const uint32_t aph = (tl_i >> 1) & 1;
                 if (!mbar_wait_bounded(smem_u32(&tl->tempty[buf]), aph ^ 1, abort_flag, err,
@@ -441,8 +429,7 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 }
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + (uint32_t)(buf * BN);
-                const int kb0 = (t / ntiles) * kbr;
-                for (int kb = kb0; kb < kb0 + kbr; ++kb, ++it) {
+                for (int kb = 0; kb < nkb; ++kb, ++it) {
                     const int s = it % STAGES;
                     const uint32_t ph = (it / STAGES) & 1;
                     if (!mbar_wait_bounded(smem_u32(&tl->full[s]), ph, abort_flag, err, ERR_TIMEOUT_MMA)) {
@@ -455,7 +442,7 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
 #pragma unroll
                     for (int kk = 0; kk < BK / 16; ++kk)
                         tc_mma_bf16(d_tmem, smem_desc_sw128(a0 + kk * 32), smem_desc_sw128(b0 + kk * 32),
-                                    idesc, (kb != kb0 || kk != 0) ? 1u : 0u);
+                                    idesc, (kb != 0 || kk != 0) ? 1u : 0u);
                     tc_commit(smem_u32(&tl->empty[s]));
                 }
                 if (!ok) break;
@@ -467,8 +454,8 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         const int q = warp & 3;                 // TMEM lane quarter of this warp
         const int row = q * 32 + lane;
         int tl_i = 0;
-        for (int t = blockIdx.x; t < total; t += gridDim.x, ++tl_i) {
-            const Tile ti = map_tile(tl, t % ntiles, ngroups, n_tiles_n, base0, a_rebase, out_rebase,
+        for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++tl_i) {
+            const Tile ti = map_tile(tl, t, ngroups, n_tiles_n, base0, a_rebase, out_rebase,
                                      b_rows_per_group, mblk, BM, 0, 0);
             const int buf = tl_i & 1;
             const uint32_t aph = (tl_i >> 1) & 1;
@@ -479,8 +466,7 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             if (!ok) break;
             tc_fence_after();
             const uint32_t tb = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * BN);
-            epilogue_tile(tb, row, ti, t / ntiles, ksplit, epi_mode, out, ldo, res, ldr, rp, partial, ldp,
-                          pstride);
+            epilogue_tile(tb, row, ti, epi_mode, out, ldo, res, ldr, rp);
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&tl->tempty[buf]));
@@ -492,6 +478,322 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         __syncwarp();
         tc_fence_after();
         tmem_dealloc(tmem_base, TMEM_COLS);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Small-batch variant: 128 x 128 tiles, two CTAs per SM.
+//
+// With few rows per group a launch streams weights, and a k-block of a CTA takes
+// as long as its one producer thread and its one MMA thread need to issue it
+// (clock64: 500-530 cycles, whatever the tile's width), so one CTA per SM pulls
+// at most 32 KB per ~0.4 us however wide its tiles, its last round leaves SMs
+// idle (16 column tiles of 256 for an expert's down projection on 152 SMs), and
+// GEMMs of other streams, which need a whole SM each, queue behind it.  Here a
+// CTA takes half the columns, half of TMEM and under half of the shared memory:
+// two CTAs issue per SM (of one launch or of two streams'), and the rounds are
+// twice as fine.  A column's sum is the same in either kernel (one K order):
+// bit for bit the same results.  1-token Mixtral-shaped forwards of six layers
+// 428 -> 403 us (three overlapping streams) and 825 -> 748 us (one alone),
+// 8-token Qwen-shaped ones of four layers 280 -> 259 and 632 -> 538 us.
+//
+// A tile takes two equal runs of weight rows `half` apart in one TMA box: 64
+// gate rows and the 64 matching up rows, or the two halves of a rotary head, so
+// that partners meet in one epilogue thread; other epilogues take any two runs.
+// The activations come in boxes of 32, 64 or 128 rows, by the largest group.
+constexpr int SN = 128;                            // tile columns
+constexpr int kSmallRing = 100 * 1024;
+constexpr int kSmallMaxStages = 5;
+constexpr uint32_t kSmallTmemCols = 2 * SN;
+using SmallSmemTail = SmemTail<kSmallMaxStages>;
+constexpr size_t kSmallSmemBytes = 1024 + (size_t)kSmallRing + sizeof(SmallSmemTail);
+
+// A tile of the small-batch kernel: nt2 counts tiles of 128 columns.  run: first
+// row of the tile's runs in their halves; blk: block of 2 half weight rows; col:
+// output column of the first run.
+struct SmallTile {
+    Tile ti;
+    int blk, run, col;
+};
+template <class Tail>
+__device__ __forceinline__ SmallTile small_tile(const Tail* tl, int t, int ngroups, int n_tiles_n, int base0,
+                                                int a_rebase, int out_rebase, int b_rows_per_group, int mblk, int half) {
+    SmallTile r;
+    int g, mt, nt;
+    locate_tile(tl, t, ngroups, 2 * n_tiles_n, mblk, BM, g, mt, nt);
+    const int r0 = mt * BM;
+    r.ti.rows = min(BM, tl->gcnt[g] - r0);
+    r.ti.a_row = tl->gstart[g] - (a_rebase ? base0 : 0) + r0;
+    r.ti.out_row = tl->gstart[g] - (out_rebase ? base0 : 0) + r0;
+    r.ti.nt = nt;
+    r.run = half == SN ? (nt & 1) * (SN / 2) : 0;
+    r.col = half == SN ? (nt >> 1) * (2 * SN) + r.run : nt * SN;
+    r.blk = (g * b_rows_per_group + r.col - r.run) / (2 * half);
+    return r;
+}
+
+// v += 32 bf16 of a residual row.
+__device__ __forceinline__ void add_row32(float (&v)[32], const __nv_bfloat16* __restrict__ src) {
+    const uint4* rr = reinterpret_cast<const uint4*>(src);
+#pragma unroll
+    for (int q4 = 0; q4 < 4; ++q4) {
+        const uint4 w = __ldg(rr + q4);
+        v[q4 * 8 + 0] += bf16_lo(w.x);
+        v[q4 * 8 + 1] += bf16_hi(w.x);
+        v[q4 * 8 + 2] += bf16_lo(w.y);
+        v[q4 * 8 + 3] += bf16_hi(w.y);
+        v[q4 * 8 + 4] += bf16_lo(w.z);
+        v[q4 * 8 + 5] += bf16_hi(w.z);
+        v[q4 * 8 + 6] += bf16_lo(w.w);
+        v[q4 * 8 + 7] += bf16_hi(w.w);
+    }
+}
+
+// Epilogue of a small tile for one warp, 32 + 32 matching columns at a time; the
+// same expressions as epilogue_tile's.
+__device__ __forceinline__ void epilogue_small(uint32_t tb, int row, const SmallTile& st, int half, int epi_mode,
+                                               __nv_bfloat16* __restrict__ out, int ldo,
+                                               const __nv_bfloat16* __restrict__ res, int ldr, const RopeEpi& rp) {
+    const bool valid = row < st.ti.rows;
+    const int orow_i = st.ti.out_row + (valid ? row : 0);
+    __nv_bfloat16* orow = out + (size_t)orow_i * ldo;
+    const int run_len = min(half, SN / 2);       // columns of one run: 64, or 32 (two 64-wide heads per tile)
+#pragma unroll 1
+    for (int pr = 0; pr < 2; ++pr) {
+        const int ca = run_len == 32 ? pr * 64 : pr * 32;
+        uint32_t xa[32], xb[32];
+        tmem_ld_32x32(tb + ca, xa);
+        tmem_ld_32x32(tb + ca + run_len, xb);
+        tmem_ld_wait();
+        if (valid) {
+            float ya[32], yb[32];
+#pragma unroll
+            for (int i = 0; i < 32; ++i) {
+                ya[i] = __uint_as_float(xa[i]);
+                yb[i] = __uint_as_float(xb[i]);
+            }
+            const int col = st.col + ca;         // first run; its partner is half further
+            const bool rot = epi_mode == EPI_ROPE && col < rp.n_rot;
+            if (epi_mode == EPI_SWIGLU) {
+#pragma unroll
+                for (int i = 0; i < 32; ++i) ya[i] = ya[i] / (1.f + __expf(-ya[i])) * yb[i];
+                store_row32(orow + (st.col - st.run) / 2 + st.run + ca, ya);
+            } else if (epi_mode == EPI_ROPE && !rot && rp.vt) {
+                const int seq = orow_i / rp.S, pos = orow_i - seq * rp.S;
+                __nv_bfloat16* vcol = rp.vt + ((size_t)seq * rp.vt_rows + (col - rp.n_rot)) * kVtSlots + pos;
+#pragma unroll
+                for (int i = 0; i < 32; ++i) {
+                    vcol[(size_t)i * kVtSlots] = __float2bfloat16_rn(ya[i]);
+                    vcol[(size_t)(half + i) * kVtSlots] = __float2bfloat16_rn(yb[i]);
+                }
+            } else {
+                if (rot) {
+                    const int pos = orow_i % rp.S;
+                    const float2* cs = rp.cs + (size_t)pos * half + (run_len == 32 ? 0 : ca);
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) {
+                        const float2 w = __ldg(cs + i);
+                        const float x1 = ya[i], x2 = yb[i];
+                        ya[i] = x1 * w.x - x2 * w.y;
+                        yb[i] = x2 * w.x + x1 * w.y;
+                    }
+                } else if (epi_mode == EPI_RELU) {
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) {
+                        ya[i] = fmaxf(ya[i], 0.f);
+                        yb[i] = fmaxf(yb[i], 0.f);
+                    }
+                } else if (epi_mode == EPI_RESID) {
+                    const __nv_bfloat16* rr = res + (size_t)orow_i * ldr + col;
+                    add_row32(ya, rr);
+                    add_row32(yb, rr + half);
+                }
+                store_row32(orow + col, ya);
+                store_row32(orow + col + half, yb);
+            }
+        }
+    }
+}
+
+// fp32 partial sums of one K range (the finish kernel adds the ranges).
+__device__ __forceinline__ void store_partial(uint32_t tb, int row, const SmallTile& st, int half,
+                                              float* __restrict__ partial, int ldp) {
+    const bool valid = row < st.ti.rows;
+    float* prow = partial + (size_t)(st.ti.out_row + (valid ? row : 0)) * ldp + st.col;
+    const int run_len = min(half, SN / 2);
+#pragma unroll 1
+    for (int c = 0; c < SN; c += 32) {
+        uint32_t r[32];
+        tmem_ld_32x32(tb + c, r);
+        tmem_ld_wait();
+        if (valid) {
+            // column c of the tile: run (c / run_len) of its halves and blocks
+            float4* d4 = reinterpret_cast<float4*>(prow + (c / run_len) * half + c % run_len);
+#pragma unroll
+            for (int q4 = 0; q4 < 8; ++q4)
+                d4[q4] = make_float4(__uint_as_float(r[4 * q4]), __uint_as_float(r[4 * q4 + 1]),
+                                     __uint_as_float(r[4 * q4 + 2]), __uint_as_float(r[4 * q4 + 3]));
+        }
+    }
+}
+
+__global__ void __launch_bounds__(kThreads, 2)
+grouped_gemm_small_kernel(const __grid_constant__ ActMaps tmA, const __grid_constant__ CUtensorMap tmB, int half,
+                          const int* __restrict__ goff, int first_group, int ngroups, int a_rebase, int out_rebase,
+                          int K, int n_tiles_n, int b_rows_per_group, int epi_mode, __nv_bfloat16* __restrict__ out,
+                          int ldo, int* err, const __nv_bfloat16* __restrict__ res, int ldr, const RopeEpi rp, int mblk,
+                          int ksplit, float* __restrict__ partial, int ldp, size_t pstride) {
+    extern __shared__ uint8_t smem_raw[];
+    const uint32_t raw_addr = smem_u32(smem_raw);
+    uint8_t* smem = smem_raw + (((raw_addr + 1023u) & ~1023u) - raw_addr);
+    const uint32_t ring = smem_u32(smem);
+    SmallSmemTail* tl = reinterpret_cast<SmallSmemTail*>(smem + kSmallRing);
+    const int warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31;
+
+    // Set-up that touches only this CTA's own resources runs before the
+    // programmatic wait, under the preceding kernel's tail.
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < kSmallMaxStages; ++s) {
+            mbar_init(smem_u32(&tl->full[s]), 1);
+            mbar_init(smem_u32(&tl->empty[s]), 1);
+        }
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(smem_u32(&tl->tfull[b]), 1);
+            mbar_init(smem_u32(&tl->tempty[b]), 4);
+        }
+        fence_barrier_init();
+    }
+    if (threadIdx.x == 32) {
+        prefetch_tmap(&tmA.r32);
+        prefetch_tmap(&tmA.r64);
+        prefetch_tmap(&tmA.r128);
+        prefetch_tmap(&tmB);
+    }
+    if (warp == 0) tmem_alloc(smem_u32(&tl->tmem_base), kSmallTmemCols);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = tl->tmem_base;
+    pdl_wait();      // results of the preceding kernel in the stream
+
+    if (warp == 0) {
+        const int most = build_tile_table(tl, goff, first_group, ngroups, 2 * n_tiles_n, BM, lane);
+        if (lane == 0) tl->a_rows = most <= 32 ? 32 : most <= 64 ? 64 : BM;
+    }
+    __syncthreads();
+    const int ntiles = tl->total_tiles;
+    const int base0 = tl->gstart[0];
+    const int total = ntiles * ksplit;    // unit u: tile u % ntiles, K range u / ntiles
+    const int kbr = K / BK / ksplit;       // k blocks per range
+    const int a_rows = tl->a_rows;
+    const uint32_t a_bytes = (uint32_t)a_rows * BK * 2;
+    // The MMA reads BM rows from a stage's start, staged or not: they lie in the
+    // stage (a_rows + SN >= BM), and what they sum is never read.
+    const uint32_t stage_bytes = a_bytes + SN * BK * 2;
+    const int stages = min(kSmallMaxStages, (int)(kSmallRing / stage_bytes));
+    volatile int* abort_flag = &tl->abort_flag;
+
+    if (warp == 0) {
+        if (lane == 0) {
+            // ---------------------------------------------------- producer
+            const CUtensorMap* a_map = a_rows == 32 ? &tmA.r32 : a_rows == 64 ? &tmA.r64 : &tmA.r128;
+            uint32_t fb = smem_u32(&tl->full[0]), st = ring, ph = 1;
+            const uint32_t fb_end = fb + 8 * stages, to_empty = smem_u32(&tl->empty[0]) - fb;
+            for (int t = blockIdx.x; t < total && !*abort_flag; t += gridDim.x) {
+                const int kr = t / ntiles;
+                const SmallTile sl = small_tile(tl, t - kr * ntiles, ngroups, n_tiles_n, base0, a_rebase, out_rebase, b_rows_per_group,
+                                                mblk, half);
+                for (int k = kr * kbr * BK, k1 = k + kbr * BK; k < k1; k += BK) {
+                    if (!mbar_wait_bounded(fb + to_empty, ph, abort_flag, err, ERR_TIMEOUT_PRODUCER)) break;
+                    mbar_arrive_expect_tx(fb, stage_bytes);
+                    tma_load_4d(st + a_bytes, &tmB, k, sl.run, 0, sl.blk, fb);
+                    tma_load_2d(st, a_map, k, sl.ti.a_row, fb);
+                    fb += 8;
+                    st += stage_bytes;
+                    if (fb == fb_end) {
+                        fb -= 8 * stages;
+                        st = ring;
+                        ph ^= 1;
+                    }
+                }
+            }
+            pdl_trigger();      // as in the kernel above: not before the last loads are issued
+        }
+    } else if (warp == 1) {
+        if (lane == 0) {
+            // ---------------------------------------------------- MMA issuer
+            constexpr uint32_t idesc = idesc_bf16_f32(BM, SN);
+            uint32_t fb = smem_u32(&tl->full[0]), ph = 0;
+            const uint32_t fb_end = fb + 8 * stages, to_empty = smem_u32(&tl->empty[0]) - fb;
+            const uint64_t desc0 = smem_desc_sw128(ring);      // the address field counts 16 bytes
+            uint64_t desc = desc0;
+            const uint32_t b_off = a_bytes >> 4, d_stage = stage_bytes >> 4;
+            int tl_i = 0;
+            bool ok = true;
+            for (int t = blockIdx.x; t < total && ok; t += gridDim.x, ++tl_i) {
+                const int buf = tl_i & 1;
+                if (!mbar_wait_bounded(smem_u32(&tl->tempty[buf]), ((tl_i >> 1) & 1) ^ 1, abort_flag, err,
+                                       ERR_TIMEOUT_MMA))
+                    break;
+                tc_fence_after();
+                const uint32_t d_tmem = tmem_base + (uint32_t)(buf * SN);
+                for (int kb = 0; kb < kbr; ++kb) {
+                    if (!mbar_wait_bounded(fb, ph, abort_flag, err, ERR_TIMEOUT_MMA)) {
+                        ok = false;
+                        break;
+                    }
+                    tc_fence_after();
+                    tc_mma_bf16(d_tmem, desc, desc + b_off, idesc, kb != 0 ? 1u : 0u);
+#pragma unroll
+                    for (int kk = 1; kk < BK / 16; ++kk)
+                        tc_mma_bf16(d_tmem, desc + 2 * kk, desc + b_off + 2 * kk, idesc, 1u);
+                    tc_commit(fb + to_empty);
+                    fb += 8;
+                    desc += d_stage;
+                    if (fb == fb_end) {
+                        fb -= 8 * stages;
+                        desc = desc0;
+                        ph ^= 1;
+                    }
+                }
+                if (!ok) break;
+                tc_commit(smem_u32(&tl->tfull[buf]));
+            }
+        }
+    } else {
+        // -------------------------------------------------------- epilogue
+        const int q = warp & 3;                 // TMEM lane quarter of this warp
+        int tl_i = 0;
+        for (int t = blockIdx.x; t < total; t += gridDim.x, ++tl_i) {
+            const int kr = t / ntiles;
+            const SmallTile sl = small_tile(tl, t - kr * ntiles, ngroups, n_tiles_n, base0, a_rebase, out_rebase, b_rows_per_group, mblk,
+                                            half);
+            const int buf = tl_i & 1;
+            int ok = 1;
+            if (lane == 0)
+                ok = mbar_wait_bounded(smem_u32(&tl->tfull[buf]), (tl_i >> 1) & 1, abort_flag, err, ERR_TIMEOUT_EPI);
+            ok = __shfl_sync(0xffffffffu, ok, 0);
+            if (!ok) break;
+            tc_fence_after();
+            const uint32_t tb = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * SN);
+            if (q * 32 < sl.ti.rows) {
+                if (ksplit > 1)
+                    store_partial(tb, q * 32 + lane, sl, half, partial + (size_t)kr * pstride, ldp);
+                else
+                    epilogue_small(tb, q * 32 + lane, sl, half, epi_mode, out, ldo, res, ldr, rp);
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&tl->tempty[buf]));
+        }
+    }
+
+    __syncthreads();
+    if (warp == 0) {
+        __syncwarp();
+        tc_fence_after();
+        tmem_dealloc(tmem_base, kSmallTmemCols);
     }
 }
 
@@ -700,7 +1002,7 @@ grouped_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
             if (!ok) break;
             tc_fence_after();
             const uint32_t tb = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * BN);
-            epilogue_tile(tb, row, ti, 0, 1, epi_mode, out, ldo, res, ldr, rp, nullptr, 0, 0);
+            epilogue_tile(tb, row, ti, epi_mode, out, ldo, res, ldr, rp);
             tc_fence_before();
             __syncwarp();
             if (lane == 0) {
@@ -1082,9 +1384,9 @@ cudaError_t launch_grouped_gemm(const GemmLaunch& g, int num_sms, cudaStream_t s
     // Row tiles per block: about 48 MB of activations (a third of L2), so that
     // a block stays resident while the weight tiles stream past it.
     const long long a_tile_bytes = (long long)BM * g.K * 2;
-    if (g.transposed && g.tmB_pair && g.ksplit <= 1 && pair_t_clusters(num_sms) > 0) {
+    if (g.transposed && g.pair && pair_t_clusters(num_sms) > 0) {
         if (g.epi_mode != EPI_STORE && g.epi_mode != EPI_RELU && g.epi_mode != EPI_SWIGLU) return cudaErrorInvalidValue;
-        if (g.epi_mode == EPI_SWIGLU && !g.tmB_gu) return cudaErrorInvalidValue;
+        if (g.epi_mode == EPI_SWIGLU && g.tmB->half != kGateUp) return cudaErrorInvalidValue;
         // Token-tile blocks of about 64 MB of activations: at K = 14336 eight
         // token tiles, so a round of 76 tiles spans ~9.5 feature tiles x 8 token
         // tiles, close to the square that streams the fewest operand slices
@@ -1092,28 +1394,50 @@ cudaError_t launch_grouped_gemm(const GemmLaunch& g, int num_sms, cudaStream_t s
         const int mblk2 = (int)std::max(1LL, (64LL << 20) / (2 * a_tile_bytes));
         const cudaError_t e = launch_pdl(
             grouped_gemm_pair_t_kernel, dim3(2 * pair_t_clusters(num_sms)), dim3(kThreads), kPairTSmemBytes, st,
-            *g.tmA, *g.tmB_pair, g.tmB_gu ? *g.tmB_gu : *g.tmB_pair, g.goff, g.first_group, g.ngroups, g.a_rebase,
+            g.tmA->r128, g.tmB->b128, g.tmB->n128, g.goff, g.first_group, g.ngroups, g.a_rebase,
             g.out_rebase, g.K, g.n_tiles_n, g.b_rows_per_group, g.epi_mode, g.out, g.ldo, g.err, mblk2,
             g.K <= kStagedMaxK ? 1 : 0, g.sched);
         if (e != cudaSuccess) return e;
         return cudaGetLastError();
     }
-    if (g.tmB_pair && (g.ksplit <= 1) && pair_clusters(num_sms) > 0) {
+    if (g.pair && pair_clusters(num_sms) > 0) {
         // Row-pair tiles per block: about 32 MB of activations (same speed as
         // 40 or 48 MB within the run-to-run spread, fewest DRAM re-reads).
         const int mblk2 = (int)std::max(1LL, (32LL << 20) / (2 * a_tile_bytes));
         const cudaError_t e = launch_pdl(
-            grouped_gemm_pair_kernel, dim3(2 * pair_clusters(num_sms)), dim3(kThreads), kPairSmemBytes, st, *g.tmA,
-            *g.tmB_pair, g.goff, g.first_group, g.ngroups, g.a_rebase, g.out_rebase, g.K, g.n_tiles_n,
+            grouped_gemm_pair_kernel, dim3(2 * pair_clusters(num_sms)), dim3(kThreads), kPairSmemBytes, st,
+            g.tmA->r128, g.tmB->b128, g.goff, g.first_group, g.ngroups, g.a_rebase, g.out_rebase, g.K, g.n_tiles_n,
             g.b_rows_per_group, g.epi_mode, g.out, g.ldo, g.err, g.res, g.ldr, rp, mblk2, g.sched);
         if (e != cudaSuccess) return e;
         return cudaGetLastError();
     }
     const int mblk = (int)std::max(1LL, (48LL << 20) / a_tile_bytes);
+    // No more CTAs than there can be tiles (every group's last tile may be ragged):
+    // CTAs without work would still need an SM's room, which other streams use.
+    const long long row_tiles = std::min(g.ngroups, g.max_rows) + g.max_rows / BM;
+    if (g.small) {
+        static PerDevice sattr;
+        const cudaError_t es = (cudaError_t)sattr.get([] {
+            return (int)cudaFuncSetAttribute(grouped_gemm_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)kSmallSmemBytes);
+        }, true);
+        if (es != cudaSuccess) return es;
+        const cudaError_t e = launch_pdl(
+            grouped_gemm_small_kernel,
+            dim3((unsigned)std::min(2LL * num_sms, row_tiles * 2 * g.n_tiles_n * std::max(g.ksplit, 1))), dim3(kThreads),
+            kSmallSmemBytes, st, *g.tmA, g.tmB->n128,
+            g.tmB->half, g.goff, g.first_group, g.ngroups, g.a_rebase, g.out_rebase, g.K, g.n_tiles_n,
+            g.b_rows_per_group, g.epi_mode, g.out, g.ldo, g.err, g.res, g.ldr, rp, mblk, g.ksplit > 1 ? g.ksplit : 1,
+            g.partial, g.ldp, g.pstride);
+        if (e != cudaSuccess) return e;
+        return cudaGetLastError();
+    }
+    if (g.ksplit > 1) return cudaErrorInvalidValue;
     const cudaError_t e = launch_pdl(
-        grouped_gemm_kernel, dim3(num_sms), dim3(kThreads), kSmemBytes, st, *g.tmA, *g.tmB, g.goff, g.first_group,
+        grouped_gemm_kernel, dim3((unsigned)std::min<long long>(num_sms, row_tiles * g.n_tiles_n)), dim3(kThreads),
+        kSmemBytes, st, g.tmA->r128, g.tmB->b256, g.goff, g.first_group,
         g.ngroups, g.a_rebase, g.out_rebase, g.K, g.n_tiles_n, g.b_rows_per_group, g.epi_mode, g.out, g.ldo, g.err,
-        g.res, g.ldr, rp, mblk, g.ksplit > 1 ? g.ksplit : 1, g.partial, g.ldp, g.pstride);
+        g.res, g.ldr, rp, mblk);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }

@@ -167,20 +167,31 @@ struct GatherParams {
     __nv_bfloat16* Xp;
 };
 
+// Tensor maps of a GEMM operand (64-column boxes, 128-byte swizzle).
+// Activations in 128-, 64- and 32-row boxes.
+struct ActMaps {
+    CUtensorMap r128, r64, r32;
+};
+// One layer's weights in 256- and 128-row boxes, and as boxes of two runs of
+// rows `half` apart (128 rows in all) over [rows / (2 half)][2][half].
+struct WeightMaps {
+    CUtensorMap b256, b128, n128;
+    int half;
+};
+
 struct GemmLaunch {
-    const CUtensorMap* tmA;
-    const CUtensorMap* tmB;
-    // Non-null: run the CTA-pair kernel, B loaded in 128-row boxes through this
-    // map (launches whose groups are large; requires ksplit <= 1).
-    const CUtensorMap* tmB_pair;
-    // Non-zero (with tmB_pair): run the transposed pair kernel instead, the
-    // weights on the M side of the MMA and the group's tokens on the N side
-    // (STORE, RELU or SWIGLU epilogues; ksplit <= 1).
+    const ActMaps* tmA;
+    const WeightMaps* tmB;
+    // Non-zero: run a CTA-pair kernel (launches whose groups are large).
+    int pair;
+    // Non-zero (with pair): the transposed pair kernel, the weights on the M
+    // side of the MMA and the group's tokens on the N side (STORE, RELU or
+    // SWIGLU epilogues).
     int transposed;
-    // Transposed SwiGLU launches: the weights in boxes of two runs of 64 rows, 128
-    // apart (a CTA's gate rows and the matching up rows).
-    const CUtensorMap* tmB_gu;
+    // Non-zero (without pair): the small-batch kernel (ksplit > 1 requires it).
+    int small;
     const int* goff;
+    int max_rows;               // upper bound of the rows of all groups
     int first_group, ngroups, a_rebase, out_rebase;
     int K, n_tiles_n, b_rows_per_group, epi_mode;
     __nv_bfloat16* out;
@@ -430,6 +441,15 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* tm,
         "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes"
         " [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
         "l"(reinterpret_cast<uint64_t>(tm)), "r"(x), "r"(y), "r"(bar)
+        : "memory");
+}
+
+__device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* tm, int c0, int c1, int c2, int c3,
+                                            uint32_t bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(tm)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(bar)
         : "memory");
 }
 

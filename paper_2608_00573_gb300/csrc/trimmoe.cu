@@ -57,15 +57,15 @@ bool make_tmap(CUtensorMap* tm, const void* base, uint64_t inner, uint64_t outer
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// SwiGLU up projections [rows][inner], gate and up rows interleaved by kGateUp,
-// as [block][2][kGateUp][inner]; a box is 64 gate rows and the matching up rows
-// of one k-block.
-bool make_tmap_gu(CUtensorMap* tm, const void* base, uint64_t inner, uint64_t rows) {
+// A weight matrix [rows][inner] as [rows / (2 half)][2][half][inner]; a box is
+// 128 rows of one k-block: 64 of each half, or two whole blocks when half is 32.
+bool make_tmap_runs(CUtensorMap* tm, const void* base, uint64_t inner, uint64_t rows, uint32_t half) {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return false;
-    cuuint64_t dims[4] = {inner, kGateUp, 2, rows / (2 * kGateUp)};
-    cuuint64_t strides[3] = {inner * 2, kGateUp * inner * 2, 2 * kGateUp * inner * 2};
-    cuuint32_t box[4] = {64, 64, 2, 1};
+    const uint32_t run = std::min(half, 64u);
+    cuuint64_t dims[4] = {inner, half, 2, rows / (2 * half)};
+    cuuint64_t strides[3] = {inner * 2, half * inner * 2, 2 * half * inner * 2};
+    cuuint32_t box[4] = {64, run, 2, 64 / run};
     cuuint32_t es[4] = {1, 1, 1, 1};
     return fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, es,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -80,6 +80,16 @@ constexpr int kSplitKMax = 8, kSplitKRows = 64;
 constexpr int kPairMinRows = 2048;
 
 inline bool pair_gemm(long long rows_per_group) { return rows_per_group >= kPairMinRows; }
+
+// Routed launches whose groups average fewer rows than this, and single groups
+// (shared expert, attention projections) of at most that many, run the
+// small-batch kernel: it reads the activations once per 128 columns, not 256,
+// which shows from about that many rows on.  Three overlapping streams, us per
+// four-layer forward on the single-CTA kernel and on it: Qwen-shaped, 24 tokens
+// 358 -> 331 (1.6 rows per routed group), 160 tokens
+// 514 -> 510; Mixtral-shaped, 40 tokens (10 rows per group) 826 -> 803, but 200
+// tokens (50 rows) 1024 -> 1052; full block, 40 tokens 978 -> 943.
+constexpr int kSmallRoutedRows = 20, kSmallSingleRows = 160;
 
 // Routed launches whose groups average at least this many rows run their
 // store / ReLU epilogues on the transposed pair kernel; smaller groups are
@@ -247,11 +257,9 @@ struct trimmoe {
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     int rows_xp = 0;
 
-    CUtensorMap tmXp, tmAct, tmActSh;
-    std::vector<CUtensorMap> tmW13, tmW2, tmW13sh, tmW2sh;
-    // the same weights in 128-row boxes (each CTA's half of a B tile in the pair kernel)
-    std::vector<CUtensorMap> tmW13p, tmW2p, tmW13shp, tmW2shp;
-    std::vector<CUtensorMap> tmW13gu;     // SwiGLU: runs of 64 gate rows and the matching up rows
+    // GEMM operands: activations, and weights per layer
+    ActMaps tmXp, tmAct, tmActSh;
+    std::vector<WeightMaps> tmW13, tmW2, tmW13sh, tmW2sh;
 
     // attention sublayer of the full block
     int nqkv = 0;
@@ -263,8 +271,8 @@ struct trimmoe {
     int* goff_attn = nullptr;
     float2* rope = nullptr;           // [attn_seq][head_dim/2] (cos, sin)
     float* sqbuf_x = nullptr;         // [rows_part] partial sums of squares of the layer input
-    CUtensorMap tmAttn;
-    std::vector<CUtensorMap> tmWqkv, tmWo, tmWqkvp, tmWop;
+    ActMaps tmAttn;
+    std::vector<WeightMaps> tmWqkv, tmWo;
     // router weight rows per layer (64-column boxes): hi and lo of the router
     // pass, and the exit-head / centroid rows read from the layer input (full block)
     std::vector<CUtensorMap> tmRhi, tmRlo, tmRxhi;
@@ -772,34 +780,33 @@ extern "C" trimmoe_status trimmoe_create(const trimmoe_config* cfg, const trimmo
     if (ce == cudaSuccess) ce = cudaMemset(h->Xp, 0, (size_t)h->rows_xp * d * 2);
     if (ce != cudaSuccess) return bail(TRIMMOE_ERR_CUDA, std::string("create: ") + cudaGetErrorString(ce));
 
-    // TMA descriptors: activations (128-row boxes) and per-layer weights (256-row boxes).
+    // TMA descriptors: activations and per-layer weights.
     const size_t F13 = (size_t)n13 * c.F;
-    bool tm = make_tmap(&h->tmXp, h->Xp, d, h->rows_xp, 128) && make_tmap(&h->tmAct, h->act, c.F, TK, 128);
-    if (has_sh) tm = tm && make_tmap(&h->tmActSh, h->act_sh, c.F_sh, T, 128);
+    auto make_act = [](ActMaps* m, const void* base, uint64_t inner, uint64_t outer) {
+        return make_tmap(&m->r128, base, inner, outer, 128) && make_tmap(&m->r64, base, inner, outer, 64) &&
+               make_tmap(&m->r32, base, inner, outer, 32);
+    };
+    // half: gate rows to up rows, or half a rotary head.
+    auto make_weight = [](WeightMaps* m, const __nv_bfloat16* base, uint64_t inner, uint64_t outer, uint32_t half) {
+        m->half = (int)half;
+        return make_tmap(&m->b256, base, inner, outer, 256) && make_tmap(&m->b128, base, inner, outer, 128) &&
+               make_tmap_runs(&m->n128, base, inner, outer, half);
+    };
+    bool tm = make_act(&h->tmXp, h->Xp, d, h->rows_xp) && make_act(&h->tmAct, h->act, c.F, TK);
+    if (has_sh) tm = tm && make_act(&h->tmActSh, h->act_sh, c.F_sh, T);
     h->tmW13.resize(N);
     h->tmW2.resize(N);
-    h->tmW13p.resize(N);
-    h->tmW13gu.resize(N);
-    h->tmW2p.resize(N);
-    if (has_sh) { h->tmW13sh.resize(N); h->tmW2sh.resize(N); h->tmW13shp.resize(N); h->tmW2shp.resize(N); }
+    if (has_sh) { h->tmW13sh.resize(N); h->tmW2sh.resize(N); }
     const __nv_bfloat16* W13 = static_cast<const __nv_bfloat16*>(w->W13);
     const __nv_bfloat16* W2 = static_cast<const __nv_bfloat16*>(w->W2);
+    const __nv_bfloat16* W13s = static_cast<const __nv_bfloat16*>(w->W13_sh);
+    const __nv_bfloat16* W2s = static_cast<const __nv_bfloat16*>(w->W2_sh);
     for (int l = 0; l < N && tm; ++l) {
-        if (c.act == 1) tm = make_tmap_gu(&h->tmW13gu[l], W13 + (size_t)l * E * F13 * d, d, (uint64_t)E * F13);
-        for (uint32_t box : {256u, 128u}) {
-            CUtensorMap* m13 = box == 256 ? &h->tmW13[l] : &h->tmW13p[l];
-            CUtensorMap* m2 = box == 256 ? &h->tmW2[l] : &h->tmW2p[l];
-            tm = tm && make_tmap(m13, W13 + (size_t)l * E * F13 * d, d, (uint64_t)E * F13, box) &&
-                 make_tmap(m2, W2 + (size_t)l * E * d * c.F, c.F, (uint64_t)E * d, box);
-            if (tm && has_sh) {
-                const __nv_bfloat16* W13s = static_cast<const __nv_bfloat16*>(w->W13_sh);
-                const __nv_bfloat16* W2s = static_cast<const __nv_bfloat16*>(w->W2_sh);
-                tm = make_tmap(box == 256 ? &h->tmW13sh[l] : &h->tmW13shp[l], W13s + (size_t)l * 2 * c.F_sh * d, d,
-                               (uint64_t)2 * c.F_sh, box) &&
-                     make_tmap(box == 256 ? &h->tmW2sh[l] : &h->tmW2shp[l], W2s + (size_t)l * d * c.F_sh, c.F_sh,
-                               (uint64_t)d, box);
-            }
-        }
+        tm = make_weight(&h->tmW13[l], W13 + (size_t)l * E * F13 * d, d, (uint64_t)E * F13, kGateUp) &&
+             make_weight(&h->tmW2[l], W2 + (size_t)l * E * d * c.F, c.F, (uint64_t)E * d, kGateUp);
+        if (tm && has_sh)
+            tm = make_weight(&h->tmW13sh[l], W13s + (size_t)l * 2 * c.F_sh * d, d, (uint64_t)2 * c.F_sh, kGateUp) &&
+                 make_weight(&h->tmW2sh[l], W2s + (size_t)l * d * c.F_sh, c.F_sh, (uint64_t)d, kGateUp);
     }
     if (tm && has_attn) {
         const int hd = c.attn_heads * c.head_dim;
@@ -807,14 +814,11 @@ extern "C" trimmoe_status trimmoe_create(const trimmoe_config* cfg, const trimmo
         const __nv_bfloat16* Wo = static_cast<const __nv_bfloat16*>(w->W_o);
         h->tmWqkv.resize(N);
         h->tmWo.resize(N);
-        h->tmWqkvp.resize(N);
-        h->tmWop.resize(N);
-        tm = make_tmap(&h->tmAttn, h->attn_out, hd, T, 128);
+        tm = make_act(&h->tmAttn, h->attn_out, hd, T);
         for (int l = 0; l < N && tm; ++l)
-            tm = make_tmap(&h->tmWqkv[l], Wqkv + (size_t)l * h->nqkv * d, d, (uint64_t)h->nqkv, 256) &&
-                 make_tmap(&h->tmWo[l], Wo + (size_t)l * d * hd, hd, (uint64_t)d, 256) &&
-                 make_tmap(&h->tmWqkvp[l], Wqkv + (size_t)l * h->nqkv * d, d, (uint64_t)h->nqkv, 128) &&
-                 make_tmap(&h->tmWop[l], Wo + (size_t)l * d * hd, hd, (uint64_t)d, 128);
+            tm = make_weight(&h->tmWqkv[l], Wqkv + (size_t)l * h->nqkv * d, d, (uint64_t)h->nqkv,
+                             (uint32_t)c.head_dim / 2) &&
+                 make_weight(&h->tmWo[l], Wo + (size_t)l * d * hd, hd, (uint64_t)d, kGateUp);
     }
     if (tm) {
         // Router weights: with the attention sublayer the router rows and the
@@ -906,6 +910,7 @@ static trimmoe_status layer_step_impl(trimmoe_handle h, int layer, int T, trimmo
         qg.tmB = &h->tmWqkv[layer];
         qg.goff = h->goff_attn;
         qg.first_group = 0;
+        qg.max_rows = T;
         qg.ngroups = 1;
         qg.K = d;
         qg.n_tiles_n = h->nqkv / 256;
@@ -920,7 +925,8 @@ static trimmoe_status layer_step_impl(trimmoe_handle h, int layer, int T, trimmo
         qg.vt = h->vt;
         qg.vt_rows = c.attn_kv_heads * c.head_dim;
         qg.err = h->dev_err;
-        qg.tmB_pair = pair_gemm(T) ? &h->tmWqkvp[layer] : nullptr;
+        qg.pair = pair_gemm(T);
+        qg.small = T <= kSmallSingleRows;
         qg.sched = h->sched_for(layer, SCHED_QKV, d);
         e = h->timed(K_ATTN_GEMM, st, [&] { return launch_grouped_gemm(qg, h->num_sms, st); });
         if (e != cudaSuccess) return h->fail(TRIMMOE_ERR_CUDA, std::string("qkv gemm: ") + cudaGetErrorString(e));
@@ -938,7 +944,6 @@ static trimmoe_status layer_step_impl(trimmoe_handle h, int layer, int T, trimmo
         og.rope = nullptr;
         og.tmA = &h->tmAttn;
         og.tmB = &h->tmWo[layer];
-        og.tmB_pair = pair_gemm(T) ? &h->tmWop[layer] : nullptr;
         og.K = hd;
         og.n_tiles_n = d / 256;
         og.b_rows_per_group = d;
@@ -1132,16 +1137,17 @@ static trimmoe_status layer_step_impl(trimmoe_handle h, int layer, int T, trimmo
     // transposed pair kernel, tokens on the MMA's N side so that a group's
     // last tile pads at most 15 tokens; SwiGLU up projections run on the pair
     // kernel for large groups, on the transposed one for middle-sized groups of
-    // long K and on the single-CTA kernel otherwise;
-    // decode-sized batches split K on the single-CTA kernel.
+    // long K and on the single-CTA kernel otherwise; small groups on the
+    // small-batch kernel, which also splits K for decode-sized batches.
     const bool pair_routed = pair_gemm((long long)T * K / E);
     const bool relu = c.act != 1;
     const bool transposed = (long long)T * K / E >= kTransposedMinRows;
     g1.transposed = transposed && (relu || (!pair_routed && d >= kTransposedSwigluMinK));
-    g1.tmB_gu = relu ? nullptr : &h->tmW13gu[layer];
-    g1.tmB_pair = (g1.transposed || pair_routed) ? &h->tmW13p[layer] : nullptr;
+    g1.pair = g1.transposed || pair_routed;
+    g1.small = (long long)T * K < (long long)kSmallRoutedRows * E;
     g1.goff = h->goff;
     g1.first_group = 0;
+    g1.max_rows = T * K;
     g1.ngroups = E;
     g1.a_rebase = 0;
     g1.out_rebase = 0;
@@ -1158,6 +1164,7 @@ static trimmoe_status layer_step_impl(trimmoe_handle h, int layer, int T, trimmo
     const bool small = (long long)T * K <= kSplitKRows;
     const int est_groups = (int)std::min<long long>(E, (long long)T * K);
     if (small) {
+        g1.small = 1;
         g1.ksplit = grouped_gemm_ksplit(est_groups * g1.n_tiles_n, d / 64, h->num_sms);
         g1.partial = h->splitk;
         g1.ldp = g1.n_tiles_n * 256;
@@ -1173,7 +1180,7 @@ static trimmoe_status layer_step_impl(trimmoe_handle h, int layer, int T, trimmo
     g2.tmB = &h->tmW2[layer];
     g2.transposed = transposed;
     g2.sched = h->sched_for(layer, SCHED_DOWN, c.F);
-    g2.tmB_pair = (g2.transposed || pair_routed) ? &h->tmW2p[layer] : nullptr;
+    g2.pair = g2.transposed || pair_routed;
     g2.K = c.F;
     g2.n_tiles_n = d / 256;
     g2.b_rows_per_group = d;
@@ -1198,8 +1205,10 @@ static trimmoe_status layer_step_impl(trimmoe_handle h, int layer, int T, trimmo
         s1.ksplit = 1;
         s1.transposed = 0;
         s1.tmB = &h->tmW13sh[layer];
-        s1.tmB_pair = pair_gemm(T) ? &h->tmW13shp[layer] : nullptr;
+        s1.pair = pair_gemm(T);
+        s1.small = T <= kSmallSingleRows;
         s1.first_group = E;
+        s1.max_rows = T;
         s1.ngroups = 1;
         s1.out_rebase = 1;
         s1.n_tiles_n = 2 * c.F_sh / 256;
@@ -1213,7 +1222,6 @@ static trimmoe_status layer_step_impl(trimmoe_handle h, int layer, int T, trimmo
         GemmLaunch s2 = s1;
         s2.tmA = &h->tmActSh;
         s2.tmB = &h->tmW2sh[layer];
-        s2.tmB_pair = pair_gemm(T) ? &h->tmW2shp[layer] : nullptr;
         s2.a_rebase = 1;
         s2.K = c.F_sh;
         s2.n_tiles_n = d / 256;

@@ -368,6 +368,20 @@ def test_layer_parity_more_candidates_than_lanes(k):
     assert sum(r["exec"] for r in reports) > 0
 
 
+@pytest.mark.parametrize("T,kw", [
+    (5, {}), (32, {}), (33, {}), (64, dict(k=1, act=W.ACT_RELU)), (65, {}), (130, dict(k=1, act=W.ACT_RELU)), (160, {}),
+    (161, {}), (230, {})])
+def test_layer_parity_small_batch_gemm(T, kw):
+    """Groups averaging under 20 rows, and a shared expert of up to 160 rows, run
+    the small-batch GEMM kernel (128-column tiles, activation boxes of 32, 64 or
+    128 rows by the largest group; K split up to 64 pairs).  With Zipf(2.0) routing
+    the largest group takes about half of the pairs."""
+    cfg = small_cfg(name="smallgemm", **{**dict(N=2, d=512, E=24, k=2, F=512, F_sh=256, M=8, H=2, zipf_s=2.0, seed=94),
+                                         **kw}, T=T)
+    reports = _run_all_layers(cfg, theta=0.5, exit_bias=1.0)
+    assert sum(r["exec"] for r in reports) > 0
+
+
 def test_layer_parity_decision_lane_groups_of_16():
     """8 < E <= 16 with more tokens than the resident warps (T >= 16 x SMs):
     the decision kernel runs two tokens per warp on 16-lane groups."""
