@@ -278,7 +278,12 @@ struct trimmoe {
     std::vector<CUtensorMap> tmRhi, tmRlo, tmRxhi;
     double flops_attn = 0.0, flops_attn_gemm = 0.0;
 
-    // host-buffer forward
+    // host-buffer forward: the hidden states, and the other token arrays in one
+    // block laid out for the call's T (those that a forward writes first, so that
+    // one copy brings them back to `back`, pinned).
+    void* host_hidden = nullptr;
+    uint8_t* host_block = nullptr;
+    uint8_t* back = nullptr;
     trimmoe_tokens dtok = {};
 
     // runtime feedback: host copies of the delay tables, window counters, scratch
@@ -1435,6 +1440,30 @@ extern "C" trimmoe_status trimmoe_forward(trimmoe_handle h, int T, trimmoe_token
     return run_forward(h, T, tok, st);
 }
 
+// Byte offsets of n tokens' state in one block, 256-byte aligned, the arrays
+// that a forward writes first.
+struct TokenBlock {
+    size_t s, Dhat, alive, last_exec, xi_last, exit_layer, written, Dbar, pJ, bytes;
+    explicit TokenBlock(size_t n) {
+        size_t at = 0;
+        auto take = [&](size_t bytes_) {
+            const size_t o = at;
+            at += (bytes_ + 255) / 256 * 256;
+            return o;
+        };
+        Dhat = take(n * 4);
+        xi_last = take(n * 4);
+        exit_layer = take(n * 2);
+        s = take(n);
+        alive = take(n);
+        last_exec = take(n);
+        written = at;
+        Dbar = take(n * 4);
+        pJ = take(n * 4);
+        bytes = at;
+    }
+};
+
 extern "C" trimmoe_status trimmoe_forward_host(trimmoe_handle h, int T, trimmoe_tokens* tok, void* stream) {
     if (!h) return TRIMMOE_ERR_ARG;
     if (T < 0 || T > h->cfg.T_max) return h->fail(TRIMMOE_ERR_ARG, "forward_host: T outside [0, T_max]");
@@ -1444,20 +1473,31 @@ extern "C" trimmoe_status trimmoe_forward_host(trimmoe_handle h, int T, trimmoe_
     DeviceGuard g(h->dev);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     h->last_stream = st;
-    const size_t Tm = h->cfg.T_max;
+    const size_t n = (size_t)T, Tm = h->cfg.T_max;
     trimmoe_tokens& dt = h->dtok;
-    if (!dt.hidden) {
+    const TokenBlock at(n);
+    if (!h->host_hidden) {
         __nv_bfloat16* hid = nullptr;
-        bool ok = h->dalloc(&hid, Tm * h->cfg.d) && h->dalloc(&dt.s, Tm) && h->dalloc(&dt.Dhat, Tm) &&
-                  h->dalloc(&dt.Dbar, Tm) && h->dalloc(&dt.pJ, Tm) && h->dalloc(&dt.alive, Tm) &&
-                  h->dalloc(&dt.last_exec, Tm) && h->dalloc(&dt.xi_last, Tm) && h->dalloc(&dt.exit_layer, Tm);
-        dt.hidden = hid;
-        if (!ok) {
-            dt.hidden = nullptr;
+        if (!h->host_block && !h->dalloc(&h->host_block, TokenBlock(Tm).bytes))
             return h->fail(TRIMMOE_ERR_OOM, "forward_host: device allocation failed");
+        if (!h->back && cudaMallocHost(reinterpret_cast<void**>(&h->back), TokenBlock(Tm).written + sizeof(int)) != cudaSuccess) {
+            cudaGetLastError();
+            h->back = nullptr;
+            return h->fail(TRIMMOE_ERR_OOM, "forward_host: pinned allocation failed");
         }
+        if (!h->dalloc(&hid, Tm * h->cfg.d)) return h->fail(TRIMMOE_ERR_OOM, "forward_host: device allocation failed");
+        h->host_hidden = hid;
     }
-    const size_t n = (size_t)T;
+    uint8_t* blk = h->host_block;
+    dt.hidden = h->host_hidden;
+    dt.s = blk + at.s;
+    dt.Dhat = reinterpret_cast<float*>(blk + at.Dhat);
+    dt.Dbar = reinterpret_cast<float*>(blk + at.Dbar);
+    dt.pJ = reinterpret_cast<float*>(blk + at.pJ);
+    dt.alive = blk + at.alive;
+    dt.last_exec = blk + at.last_exec;
+    dt.xi_last = reinterpret_cast<float*>(blk + at.xi_last);
+    dt.exit_layer = reinterpret_cast<int16_t*>(blk + at.exit_layer);
     struct Cp { void* dst; const void* src; size_t bytes; };
     const Cp in[] = {{dt.hidden, tok->hidden, n * h->cfg.d * 2}, {dt.s, tok->s, n}, {dt.Dhat, tok->Dhat, n * 4},
                      {dt.Dbar, tok->Dbar, n * 4}, {dt.pJ, tok->pJ, n * 4}, {dt.alive, tok->alive, n},
@@ -1470,12 +1510,24 @@ extern "C" trimmoe_status trimmoe_forward_host(trimmoe_handle h, int T, trimmoe_
         trimmoe_status s = run_forward(h, T, &dt, st);
         if (s != TRIMMOE_OK) return s;
     }
-    for (const Cp& c : in)
-        if (cudaMemcpyAsync(const_cast<void*>(c.src), c.dst, c.bytes, cudaMemcpyDeviceToHost, st) != cudaSuccess)
-            return h->fail(TRIMMOE_ERR_CUDA, "forward_host: device-to-host copy failed");
+    // Back: the hidden states, the written arrays in one copy and the error word
+    // (Dbar and pJ are only read); the arrays are handed out once the stream is done.
+    // (Nine copies and a blocking one for the error word took 18-25 us more:
+    // 777-token Switch-shaped forwards of four layers 406 -> 387 us.)
+    int* derr_back = reinterpret_cast<int*>(h->back);
+    uint8_t* back = h->back + sizeof(int);
+    if (cudaMemcpyAsync(tok->hidden, dt.hidden, n * h->cfg.d * 2, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+        cudaMemcpyAsync(back, blk, at.written, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+        cudaMemcpyAsync(derr_back, h->dev_err, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess)
+        return h->fail(TRIMMOE_ERR_CUDA, "forward_host: device-to-host copy failed");
     if (cudaStreamSynchronize(st) != cudaSuccess) return h->fail(TRIMMOE_ERR_CUDA, "forward_host: sync failed");
-    int derr = 0;
-    cudaMemcpy(&derr, h->dev_err, sizeof(int), cudaMemcpyDeviceToHost);
+    std::memcpy(tok->s, back + at.s, n);
+    std::memcpy(tok->Dhat, back + at.Dhat, n * 4);
+    std::memcpy(tok->alive, back + at.alive, n);
+    std::memcpy(tok->last_exec, back + at.last_exec, n);
+    std::memcpy(tok->xi_last, back + at.xi_last, n * 4);
+    std::memcpy(tok->exit_layer, back + at.exit_layer, n * 2);
+    const int derr = *derr_back;
     if (derr) return h->fail(TRIMMOE_ERR_DEVICE_TIMEOUT, "forward_host: a kernel timed out waiting");
     return TRIMMOE_OK;
 }
@@ -1796,5 +1848,6 @@ extern "C" void trimmoe_destroy(trimmoe_handle h) {
     if (h->ev_join) cudaEventDestroy(h->ev_join);
     if (h->aux) cudaStreamDestroy(h->aux);
     for (void* p : h->allocs) cudaFree(p);
+    if (h->back) cudaFreeHost(h->back);
     delete h;
 }

@@ -183,6 +183,33 @@ def test_forward_host_equals_device_forward():
     eng.close()
 
 
+def test_forward_host_with_changing_batches():
+    """The handle lays the token arrays out for each call's T: batches of other
+    sizes, replayed ones among them (graphs), leave each other's results alone,
+    and Dbar and pJ (only read) keep their values.  Pageable arrays work too."""
+    import torch
+    cfg = SMALL["swiglu_k2_renorm_h2"]
+    small = W.make_small_weights(cfg, calib={"exit_bias": [1.0] * cfg.N})
+    tables = W.make_tables(cfg, small["W_r"], calib={"theta": [0.9] * cfg.N})
+    eng = B.Engine(cfg, tables, small, W.make_expert_weights_host(cfg), T_max=333, graphs=True)
+    stream = torch.cuda.Stream()
+    for T, pinned in ((333, True), (1, True), (77, False), (77, True), (77, True), (333, False)):
+        tok = W.make_tokens(cfg, T=T, seed_offset=T)
+        dev = eng.tokens_to_device(tok)
+        torch.cuda.synchronize()
+        eng.forward(dev)                       # the legacy stream: plain launches
+        torch.cuda.synchronize()
+        want = B.Engine.tokens_to_host(dev)
+        host = {k: v.cpu() for k, v in eng.tokens_to_device(tok).items()}
+        if pinned:
+            host = {k: v.pin_memory() for k, v in host.items()}
+        eng.forward_host(host, stream=stream)
+        got = B.Engine.tokens_to_host(host)
+        for k in want:
+            assert np.array_equal(want[k], got[k]), (T, k)
+    eng.close()
+
+
 def test_stats_counters_consistent():
     import torch
     cfg = SMALL["swiglu_k2_renorm_h2"]
