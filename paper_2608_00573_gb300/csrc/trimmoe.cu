@@ -91,11 +91,21 @@ inline bool pair_gemm(long long rows_per_group) { return rows_per_group >= kPair
 // tokens (50 rows) 1024 -> 1052; full block, 40 tokens 978 -> 943.
 constexpr int kSmallRoutedRows = 20, kSmallSingleRows = 160;
 
-// Routed launches whose groups average at least this many rows run their
-// store / ReLU epilogues on the transposed pair kernel; smaller groups are
+// Routed launches run their store / ReLU epilogues on the transposed pair
+// kernel when their groups average this many rows; smaller groups are
 // weight-streaming bound, and its 256-feature pair tiles would leave a ragged
 // last round (Mixtral-shaped decode at 256 tokens: 15.2 -> 15.6 ms per step).
-constexpr int kTransposedMinRows = 256;
+// Batches of few rows in all, whose tiles fill only a round or two, already gain
+// from the smaller number of rows (us per layer: Mixtral-shaped, 520 tokens, 130
+// rows per group 585 -> 547, 1000 tokens 677 -> 669; Switch-shaped, 1100 tokens
+// 80.1 -> 76.5, 1900 tokens 87.6 -> 79.8); with many groups of that size the
+// row kernel's rate decides (Qwen-shaped, 2100 tokens, 140 rows per group in 60
+// groups: 378 -> 385).
+constexpr int kTransposedMinRows = 256, kTransposedMinRowsFew = 128, kTransposedFewRows = 4096;
+
+inline bool transposed_gemm(long long rows, int groups) {
+    return rows >= (long long)(rows <= kTransposedFewRows ? kTransposedMinRowsFew : kTransposedMinRows) * groups;
+}
 
 // SwiGLU up projections of those groups run there too from this K on (and below
 // kPairMinRows rows per group, where the row-pair kernel's padding weighs less
@@ -1137,7 +1147,7 @@ static trimmoe_status layer_step_impl(trimmoe_handle h, int layer, int T, trimmo
     GemmLaunch g1{};
     g1.tmA = &h->tmXp;
     g1.tmB = &h->tmW13[layer];
-    // Routed experts: with at least kTransposedMinRows rows per expert the
+    // Routed experts: with enough rows per expert (transposed_gemm) the
     // down projection (and the up projection of ReLU experts) runs on the
     // transposed pair kernel, tokens on the MMA's N side so that a group's
     // last tile pads at most 15 tokens; SwiGLU up projections run on the pair
@@ -1146,7 +1156,7 @@ static trimmoe_status layer_step_impl(trimmoe_handle h, int layer, int T, trimmo
     // small-batch kernel, which also splits K for decode-sized batches.
     const bool pair_routed = pair_gemm((long long)T * K / E);
     const bool relu = c.act != 1;
-    const bool transposed = (long long)T * K / E >= kTransposedMinRows;
+    const bool transposed = transposed_gemm((long long)T * K, E);
     g1.transposed = transposed && (relu || (!pair_routed && d >= kTransposedSwigluMinK));
     g1.pair = g1.transposed || pair_routed;
     g1.small = (long long)T * K < (long long)kSmallRoutedRows * E;

@@ -362,10 +362,11 @@ def test_layer_parity_transposed_pair_gemm(name, kw):
 @pytest.mark.parametrize("name,kw", [
     ("F384_T1100", dict(E=8, k=2, F=384, T=1100, zipf_s=1.0)),
     ("F128_T515", dict(E=2, k=1, F=128, T=515, zipf_s=0.3)),
+    ("F256_T530", dict(E=4, k=1, F=256, T=530, zipf_s=1.0)),
 ])
 def test_layer_parity_transposed_swiglu(name, kw):
-    """SwiGLU up projections with K = d >= 4096 and groups averaging 256 to 2047
-    rows run on the transposed CTA-pair kernel (gate and up lanes swapped
+    """SwiGLU up projections with K = d >= 4096 and groups averaging 256 (128 for
+    few rows in all) to 2047 rows run on the transposed CTA-pair kernel (gate and up lanes swapped
     between warps): token tiles from a few rows to 256 with tails inside a
     16-token step, one and three blocks of 128 features."""
     cfg = small_cfg(name=name, N=2, d=4096, M=10, H=3, seed=97, **kw)
