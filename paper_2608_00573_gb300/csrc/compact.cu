@@ -64,23 +64,37 @@ __global__ void __launch_bounds__(kChunk) scatter_kernel(const CompactParams p) 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nb = p.E + 1;
     for (int i = threadIdx.x; i < kScatWarps * nb; i += blockDim.x) run[i / nb][i % nb] = 0;
-    // Chunk base and total per bucket: a warp per bucket, lanes over chunks.
-    for (int e = warp; e < (kSingle ? 0 : nb); e += kScatWarps) {
-        int pre = 0, all = 0;
+    // Chunk base and total per bucket: a warp per bucket, lanes over chunks, four
+    // buckets' reads in flight (one at a time, 61 buckets were eight rounds of
+    // latency in a row: Qwen-shaped layer of 2100
+    // tokens 378.5 -> 376.0 us, Switch-shaped of 4096 90.2 -> 89.5 us).
+    constexpr int kB = 4;
+    for (int e0 = warp; e0 < (kSingle ? 0 : nb); e0 += kB * kScatWarps) {
+        int pre[kB], all[kB];
+#pragma unroll
+        for (int u = 0; u < kB; ++u) pre[u] = all[u] = 0;
         for (int b0 = 0; b0 < p.nblk; b0 += 32) {
             const int b = b0 + lane;
-            const int c = b < p.nblk ? p.blk_counts[b * nb + e] : 0;
-            all += c;
-            pre += b < (int)blockIdx.x ? c : 0;
+            int c[kB];
+#pragma unroll
+            for (int u = 0; u < kB; ++u) {
+                const int e = e0 + u * kScatWarps;
+                c[u] = b < p.nblk && e < nb ? p.blk_counts[b * nb + e] : 0;
+            }
+#pragma unroll
+            for (int u = 0; u < kB; ++u) {
+                all[u] += c[u];
+                pre[u] += b < (int)blockIdx.x ? c[u] : 0;
+            }
         }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            all += __shfl_xor_sync(0xffffffffu, all, o);
-            pre += __shfl_xor_sync(0xffffffffu, pre, o);
-        }
-        if (lane == 0) {
-            cbase[e] = pre;
-            total[e] = all;
+        for (int u = 0; u < kB; ++u) {
+            const int e = e0 + u * kScatWarps;
+            const int ta = __reduce_add_sync(0xffffffffu, all[u]), tp = __reduce_add_sync(0xffffffffu, pre[u]);
+            if (lane == 0 && e < nb) {
+                cbase[e] = tp;
+                total[e] = ta;
+            }
         }
     }
     __syncthreads();
