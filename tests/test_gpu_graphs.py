@@ -140,3 +140,40 @@ def test_graph_follows_feedback_updates():
     plain.close()
     graph.close()
     torch.cuda.synchronize()
+
+
+def test_caller_capture_with_shared_expert():
+    """A caller's own capture of a forward and of a layer step takes in the side
+    stream that runs the shared expert's GEMMs: replays equal plain launches, and
+    the handle stays usable on other streams."""
+    import torch
+    cfg = small_cfg(name="cap", N=3, d=512, E=8, k=2, F=256, F_sh=384, T=300, M=8, H=3, seed=93)
+    eng, om, tables, small, experts = make_engine(cfg, T_max=300, theta=0.9, exit_bias=1.0)
+    tok = W.make_tokens(cfg)
+    init = eng.tokens_to_device(tok)
+    want = {k: v.clone() for k, v in init.items()}
+    eng.forward(want)
+    eng.layer_step(1, want)
+    torch.cuda.synchronize()
+    work = {k: v.clone() for k, v in init.items()}
+    stream = torch.cuda.Stream()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=stream):
+        eng.forward(work, stream=stream)
+        eng.layer_step(1, work, stream=stream)
+    for _ in range(2):
+        for k in work:
+            work[k].copy_(init[k])
+        g.replay()
+        torch.cuda.synchronize()
+        for k in work:
+            assert torch.equal(work[k], want[k]), k
+    again = {k: v.clone() for k, v in init.items()}
+    with torch.cuda.stream(stream):
+        eng.forward(again, stream=stream)
+        eng.layer_step(1, again, stream=stream)
+    torch.cuda.synchronize()
+    for k in again:
+        assert torch.equal(again[k], want[k]), k
+    assert eng.stats()["status"] == 0
+    eng.close()
