@@ -1,7 +1,7 @@
 // Host runtime of the C ABI declared in include/trimmoe.h: validation, the
 // candidate lists V_{l,r} with their losses Q (Eq. 3), workspaces, TMA
 // descriptors, and the per-layer launch sequence
-//   decide -> compact -> gather -> FFN gate/up -> FFN down -> combine
+//   router -> decide -> compact + gather -> FFN gate/up -> FFN down -> combine
 // (the per-layer body of Algorithm 2 plus the MoE computation it gates).
 #include <algorithm>
 #include <cmath>
@@ -10,6 +10,7 @@
 #include <cstring>
 #include <limits>
 #include <mutex>
+#include <new>
 #include <string>
 #include <utility>
 #include <vector>
@@ -291,10 +292,11 @@ struct trimmoe {
 
     // host-buffer forward: the hidden states, and the other token arrays in one
     // block laid out for the call's T (those that a forward writes first, so that
-    // one copy brings them back to `back`, pinned).
+    // one copy brings them back to `back`).
     void* host_hidden = nullptr;
     uint8_t* host_block = nullptr;
     uint8_t* back = nullptr;
+    bool back_pinned = false;
     trimmoe_tokens dtok = {};
 
     // runtime feedback: host copies of the delay tables, window counters, scratch
@@ -1509,10 +1511,14 @@ extern "C" trimmoe_status trimmoe_forward_host(trimmoe_handle h, int T, trimmoe_
         __nv_bfloat16* hid = nullptr;
         if (!h->host_block && !h->dalloc(&h->host_block, TokenBlock(Tm).bytes))
             return h->fail(TRIMMOE_ERR_OOM, "forward_host: device allocation failed");
-        if (!h->back && cudaMallocHost(reinterpret_cast<void**>(&h->back), TokenBlock(Tm).written + sizeof(int)) != cudaSuccess) {
-            cudaGetLastError();
-            h->back = nullptr;
-            return h->fail(TRIMMOE_ERR_OOM, "forward_host: pinned allocation failed");
+        if (!h->back) {
+            const size_t bytes = TokenBlock(Tm).written + sizeof(int);
+            h->back_pinned = cudaMallocHost(reinterpret_cast<void**>(&h->back), bytes) == cudaSuccess;
+            if (!h->back_pinned) {             // pageable memory does too
+                cudaGetLastError();
+                h->back = new (std::nothrow) uint8_t[bytes];
+            }
+            if (!h->back) return h->fail(TRIMMOE_ERR_OOM, "forward_host: host allocation failed");
         }
         if (!h->dalloc(&hid, Tm * h->cfg.d)) return h->fail(TRIMMOE_ERR_OOM, "forward_host: device allocation failed");
         h->host_hidden = hid;
@@ -1877,6 +1883,7 @@ extern "C" void trimmoe_destroy(trimmoe_handle h) {
     if (h->ev_join) cudaEventDestroy(h->ev_join);
     if (h->aux) cudaStreamDestroy(h->aux);
     for (void* p : h->allocs) cudaFree(p);
-    if (h->back) cudaFreeHost(h->back);
+    if (h->back_pinned) cudaFreeHost(h->back);
+    else delete[] h->back;
     delete h;
 }
