@@ -675,9 +675,9 @@ __global__ void __launch_bounds__(kWarps * 32, KEEP ? 4 : 7) decide_kernel(const
 // One look-ahead table for Dbar = Dbar[0]: layer l, interval iv (R =
 // thr[iv - 1], or -inf for iv = 0), depth top (levels l + top .. l + 1), each
 // entry by one thread with the same operation order as the per-token path
-// above, written to out.  A block has a thread per entry (up to 1024): each
-// entry is a chain of dependent loads and roundings, so a table is
-// latency-bound.  Called by whole blocks.
+// above, written to out.  Each entry is a chain of dependent loads and
+// roundings, so a table is latency-bound; blockDim.x threads share the entries.
+// Called by whole blocks.
 __device__ __forceinline__ void lookahead_table(const DecideParams& p, int l, const float* thr, int iv, int top,
                                                 float* out) {
     extern __shared__ float smem[];
@@ -790,12 +790,21 @@ cudaError_t launch_lookahead_shared(const DecideParams& p, int n_depth, cudaStre
 }
 
 cudaError_t launch_lookahead_all(const DecideParams& p, const LaLayer* layers, int n_layers, int max_thr,
-                                 int max_depth, cudaStream_t st) {
+                                 int max_depth, int n_tables, int num_sms, cudaStream_t st) {
     if (p.T <= 0 || n_layers <= 0 || max_depth <= 0) return cudaSuccess;
     const size_t MC = (size_t)p.tab.max_layer_cand;
     const size_t smem = (2 * (size_t)p.M * p.E + 2 * MC) * sizeof(float) + ((MC + 3) / 4) * 2 * sizeof(float);
+    // A thread per entry for up to three tables per SM; above that 256 threads,
+    // the entries in turns.  The launch alone takes as long either way (591
+    // tables of 600 entries: 32 us); with many tables the smaller blocks leave
+    // threads and registers of every SM to what runs beside it (three
+    // overlapping streams of four-layer Qwen-shaped forwards of 8 tokens
+    // 247 -> 239 us a forward, of 2 tokens 198 -> 190).  With fewer there is
+    // room anyway, and a block of 256 only takes longer (123 tables, two
+    // layers: 103.9 -> 105.6 us a forward, one alone 222 -> 227; 360 tables,
+    // three layers: 164.4 -> 163.1, one alone 347 -> 355).
     const int ME = p.M * p.E;
-    const int threads = std::min(1024, std::max(256, (ME + 31) / 32 * 32));
+    const int threads = n_tables > 3 * num_sms ? 256 : std::min(1024, std::max(256, (ME + 31) / 32 * 32));
     lookahead_all_kernel<<<dim3(max_thr + 1, max_depth, n_layers), threads, smem, st>>>(p, layers);
     return cudaGetLastError();
 }

@@ -285,12 +285,13 @@ size_t decide_la_scratch_floats(int E, int M, int max_layer_cand, int num_sms);
 cudaError_t launch_lookahead_shared(const DecideParams& p, int n_depth, cudaStream_t st);
 // Placement of one layer's shared look-ahead tables when every layer's tables
 // are computed in one launch: thresholds p.thr[thr_off .. thr_off + n_thr),
-// n_depth depths, tables from p.phi_tabs_out + tab_off.
+// n_depth depths, tables from p.phi_tabs_out + tab_off.  n_tables: their number
+// over all layers.
 struct LaLayer {
     int thr_off, n_thr, n_depth, tab_off;
 };
 cudaError_t launch_lookahead_all(const DecideParams& p, const LaLayer* layers, int n_layers, int max_thr,
-                                 int max_depth, cudaStream_t st);
+                                 int max_depth, int n_tables, int num_sms, cudaStream_t st);
 cudaError_t launch_compact(const CompactParams& p, cudaStream_t st);
 cudaError_t launch_gather(const int32_t* perm, const int32_t* goff, const GatherParams& q, int max_rows, int num_sms,
                           cudaStream_t st);

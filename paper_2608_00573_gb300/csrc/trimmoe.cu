@@ -229,7 +229,7 @@ struct trimmoe {
     bool la_all = false, tabs_ready = false;
     std::vector<LaLayer> h_la;
     LaLayer* la_layers = nullptr;
-    int la_max_thr = 0, la_max_depth = 0;
+    int la_max_thr = 0, la_max_depth = 0, la_tables = 0;
     float* dbar_shared = nullptr;     // [1]
     float* cnorm = nullptr;           // [N][K_c] centroid norms
     int16_t* lhat = nullptr;          // [N][K_c] rounded average exit layers
@@ -636,6 +636,7 @@ extern "C" trimmoe_status trimmoe_create(const trimmoe_config* cfg, const trimmo
             if (L.n_depth > 0) {
                 h->la_max_thr = std::max(h->la_max_thr, L.n_thr);
                 h->la_max_depth = std::max(h->la_max_depth, L.n_depth);
+                h->la_tables += L.n_depth * (L.n_thr + 1);
             }
         }
         h->la_all = total > 0 && total <= kMaxAllTabFloats;
@@ -1354,7 +1355,8 @@ static bool build_all_tables(trimmoe_handle h, int T, const trimmoe_tokens* tok,
     dp.tab.PT = h->PT;
     dp.tab.eps = h->eps;
     *err = h->timed(K_DECIDE, st, [&] {
-        return launch_lookahead_all(dp, h->la_layers, c.N, h->la_max_thr, h->la_max_depth, st);
+        return launch_lookahead_all(dp, h->la_layers, c.N, h->la_max_thr, h->la_max_depth, h->la_tables, h->num_sms,
+                                    st);
     });
     if (*err != cudaSuccess) return false;
     h->launches += 1;

@@ -491,6 +491,29 @@ def test_forward_tables_for_all_layers_equal_per_layer_tables(n_centroids, T):
     eng.close()
 
 
+@pytest.mark.parametrize("N,H,E,M", [(2, 2, 60, 10), (6, 3, 31, 9), (6, 3, 64, 16), (6, 2, 8, 10)])
+def test_forward_tables_few_and_many(N, H, E, M):
+    """Tables of at most and of more entries than a block's threads, and few and
+    many of them: a forward that reads them equals layer steps in which every
+    token computes its own, bit for bit."""
+    import torch
+    cfg = small_cfg(name=f"tabs_{N}_{E}", N=N, d=256, E=E, k=2, F=128, T=200, M=M, H=H, zipf_s=1.0, seed=131)
+    eng, om, tables, small, experts = make_engine(cfg, theta=0.6, exit_bias=1.0)
+    tok = W.make_tokens(cfg)
+    a, b = eng.tokens_to_device(tok), eng.tokens_to_device(tok)
+    eng.reset_stats()
+    eng.forward(a)
+    torch.cuda.synchronize()
+    assert eng.stats()["lookahead_shared"] > 0
+    for l in range(cfg.N):
+        eng.layer_step(l, b)
+    torch.cuda.synchronize()
+    ha, hb = B.Engine.tokens_to_host(a), B.Engine.tokens_to_host(b)
+    for key in ha:
+        assert np.array_equal(ha[key], hb[key]), key
+    eng.close()
+
+
 @pytest.mark.parametrize("n_centroids", [0, 32])
 def test_shared_lookahead_tables_with_mixed_budgets(n_centroids):
     """Many tokens of one budget read the look-ahead table (Eq. 39) of their
