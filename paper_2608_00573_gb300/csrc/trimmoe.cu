@@ -377,14 +377,22 @@ struct trimmoe {
         return e;
     }
 
+    // Adds the time between a launch's two events once both have passed.  The
+    // events of one forward lie on several streams, so each pair is waited for by
+    // itself.  A failure is cleared: the next launch would report it as its own.
+    void add_elapsed(const std::pair<std::pair<cudaEvent_t, cudaEvent_t>, int>& pe) {
+        float t = 0.f;
+        if (cudaEventSynchronize(pe.first.second) == cudaSuccess &&
+            cudaEventElapsedTime(&t, pe.first.first, pe.first.second) == cudaSuccess)
+            ms[pe.second] += t;
+        else
+            cudaGetLastError();
+    }
+
     // Adds the kernel times of a finished graph replay (waits for it if needed).
     void read_graph_inst(GraphInst& gi) {
         if (!gi.pending) return;
-        if (!gi.evs.empty()) cudaEventSynchronize(gi.evs.back().first.second);
-        for (auto& pe : gi.evs) {
-            float t = 0.f;
-            if (cudaEventElapsedTime(&t, pe.first.first, pe.first.second) == cudaSuccess) ms[pe.second] += t;
-        }
+        for (auto& pe : gi.evs) add_elapsed(pe);
         gi.pending = false;
     }
 
@@ -405,8 +413,7 @@ struct trimmoe {
     void drain_events() {
         for (GraphInst& gi : fg.inst) read_graph_inst(gi);
         for (auto& pe : ev_pending) {
-            float t = 0.f;
-            if (cudaEventElapsedTime(&t, pe.first.first, pe.first.second) == cudaSuccess) ms[pe.second] += t;
+            add_elapsed(pe);
             ev_free.push_back(pe.first.first);
             ev_free.push_back(pe.first.second);
         }

@@ -1,0 +1,76 @@
+"""Stream and event handling of the runtime, on the CPU: the host object linked
+with a CUDA runtime that runs nothing but keeps the order of launches, event
+records and event waits (fake_cuda.cpp)."""
+import ctypes as C
+import os
+import subprocess
+
+import pytest
+
+from paper_2608_00573_gb300 import binding as B
+from paper_2608_00573_gb300 import build as BUILD
+from paper_2608_00573_gb300 import workload as W
+from tests.oracle_helpers import small_cfg
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+class Stream:
+    """What the binding reads of a torch stream."""
+
+    def __init__(self, fake, ptr=0x500, priority=0):
+        self.cuda_stream = ptr
+        fake.fake_stream(C.c_void_p(ptr), priority)
+
+
+@pytest.fixture(scope="module")
+def fake_path(tmp_path_factory):
+    BUILD.build()
+    out = str(tmp_path_factory.mktemp("fake") / "libtrimmoe_fake.so")
+    inc = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(BUILD.nvcc()))), "include")
+    subprocess.check_call(["g++", "-shared", "-fPIC", "-std=c++17", "-Wl,-Bsymbolic", "-I", inc,
+                           os.path.join(HERE, "fake_cuda.cpp"), os.path.join(BUILD.BUILD, "trimmoe.o"), "-o", out, "-ldl"])
+    return out
+
+
+@pytest.fixture
+def fake(fake_path, monkeypatch):
+    monkeypatch.setattr(B, "LIB_PATH", fake_path)
+    monkeypatch.setattr(B, "_lib", None)
+    L = B.lib()
+    L.fake_launch_name.restype = C.c_char_p
+    L.fake_launch_stream.restype = C.c_void_p
+    L.fake_launch_stream.argtypes = L.fake_launch_name.argtypes = [C.c_int]
+    L.fake_reset()
+    return L
+
+
+def engine(cfg, **kw):
+    small = W.make_small_weights(cfg, calib={"exit_bias": [1.0] * cfg.N})
+    tables = W.make_tables(cfg, small["W_r"], calib={"theta": [0.6] * cfg.N})
+    eng = B.Engine(cfg, tables, small, W.make_expert_weights_host(cfg), T_max=cfg.T, device="cpu", **kw)
+    return eng, eng.tokens_to_device(W.make_tokens(cfg))
+
+
+def launches(fake):
+    return [(fake.fake_launch_name(i).decode(), fake.fake_launch_stream(i)) for i in range(fake.fake_launches())]
+
+
+def shared_cfg(**kw):
+    return small_cfg(**{**dict(name="streams", N=2, d=256, E=4, k=2, F=128, F_sh=256, T=40, M=4, H=2, seed=71), **kw})
+
+
+@pytest.mark.parametrize("profile", [1, 2])
+def test_replayed_launch_times_are_all_read(fake, profile):
+    """Replays in a row without a host wait, then another batch size: every GEMM
+    launch that is counted is timed, and reading the times leaves no error for
+    the next launch to report."""
+    eng, tok = engine(shared_cfg(), profile=profile, graphs=True)
+    st = Stream(fake)
+    for T in (40, 24, 40):
+        for _ in range(5):          # plain, then replays of both instances
+            eng.forward(tok, T=T, stream=st)
+    s = eng.stats()
+    assert s["n_gemm_up"] == s["n_gemm_down"] == 15 * 4
+    assert s["ms_gemm_up"] + s["ms_gemm_down"] == s["n_gemm_up"] + s["n_gemm_down"]
+    eng.close()
