@@ -77,6 +77,9 @@ enum { TRIMMOE_EXEC = 0, TRIMMOE_SKIP = 1, TRIMMOE_EXIT = 2, TRIMMOE_DEAD = 3 };
  *  profile: 1 = record CUDA events around each kernel launch (trimmoe_stats
  *  then reports per-kernel device time); 2 = around the grouped GEMM launches
  *  only (each event pair inside a replayed graph costs a few microseconds);
+ *  either way a shared expert's GEMMs run on the caller's stream in turn with
+ *  the routed ones instead of beside them, so that the launches' times add up
+ *  (a forward then takes longer than with 0, with the same results);
  *  norm_eps: epsilon of the pre-FFN RMSNorm (used when W_norm != NULL);
  *  n_centroids: K_c centroids per layer for the token-similarity exit-point
  *  prediction of Eq. (36) (0 = off, at most 256);

@@ -377,9 +377,9 @@ struct trimmoe {
         return e;
     }
 
-    // Adds the time between a launch's two events once both have passed.  The
-    // events of one forward lie on several streams, so each pair is waited for by
-    // itself.  A failure is cleared: the next launch would report it as its own.
+    // Adds the time between a launch's two events once both have passed: each pair
+    // is waited for by itself, whatever stream it was recorded on.  A failure is
+    // cleared: the next launch would report it as its own.
     void add_elapsed(const std::pair<std::pair<cudaEvent_t, cudaEvent_t>, int>& pe) {
         float t = 0.f;
         if (cudaEventSynchronize(pe.first.second) == cudaSuccess &&
@@ -1202,11 +1202,16 @@ static trimmoe_status layer_step_impl(trimmoe_handle h, int layer, int T, trimmo
     // in its last round (8 column tiles of the shared down projection on 152 SMs
     // at a few tokens): Qwen-shaped, 8-token forwards of four layers 542 -> 478 us
     // alone and 261 -> 247 us with three streams, a layer of 700 tokens 308 -> 282
-    // us, of 2000 387 -> 366 us, of 8192 831 -> 807 us.
+    // us, of 2000 387 -> 366 us, of 8192 831 -> 807 us.  With profiling they stay
+    // on the caller's stream: the times of launches that share the SMs would not
+    // add up.
+    const bool sh_aside = has_sh && c.profile == 0;
     if (has_sh) {
-        cudaStream_t ss = h->aux;
-        e = cudaEventRecord(h->ev_fork, st);
-        if (e == cudaSuccess) e = cudaStreamWaitEvent(ss, h->ev_fork, 0);
+        cudaStream_t ss = sh_aside ? h->aux : st;
+        if (sh_aside) {
+            e = cudaEventRecord(h->ev_fork, st);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(ss, h->ev_fork, 0);
+        }
         if (e != cudaSuccess) return h->fail(TRIMMOE_ERR_CUDA, std::string("shared fork: ") + cudaGetErrorString(e));
         GemmLaunch s1 = g1;
         s1.ksplit = 1;
@@ -1242,7 +1247,7 @@ static trimmoe_status layer_step_impl(trimmoe_handle h, int layer, int T, trimmo
         h->n_gemm_up++;
         h->n_gemm_down++;
         h->launches += 2;
-        e = cudaEventRecord(h->ev_join, ss);
+        if (sh_aside) e = cudaEventRecord(h->ev_join, ss);
         if (e != cudaSuccess) return h->fail(TRIMMOE_ERR_CUDA, std::string("shared join: ") + cudaGetErrorString(e));
     }
 
@@ -1276,7 +1281,7 @@ static trimmoe_status layer_step_impl(trimmoe_handle h, int layer, int T, trimmo
     // router, decide, compaction (count, scatter, gather, or one), gate/up GEMM, down GEMM
     // (+ look-ahead tables, split-K finishes)
     h->launches += (fused ? 5 : 7) + (tabs_here ? 1 : 0) + (g1.ksplit > 1 ? 1 : 0) + (g2.ksplit > 1 ? 1 : 0);
-    if (has_sh) {
+    if (sh_aside) {
         e = cudaStreamWaitEvent(st, h->ev_join, 0);
         if (e != cudaSuccess) return h->fail(TRIMMOE_ERR_CUDA, std::string("shared join: ") + cudaGetErrorString(e));
     }

@@ -74,3 +74,17 @@ def test_replayed_launch_times_are_all_read(fake, profile):
     assert s["n_gemm_up"] == s["n_gemm_down"] == 15 * 4
     assert s["ms_gemm_up"] + s["ms_gemm_down"] == s["n_gemm_up"] + s["n_gemm_down"]
     eng.close()
+
+
+@pytest.mark.parametrize("profile", [0, 1, 2])
+def test_timed_launches_do_not_overlap(fake, profile):
+    """With profiling every GEMM launch is on the caller's stream, so that the
+    times of the launches add up; without, the shared expert's two run beside
+    the routed ones."""
+    cfg = shared_cfg()
+    eng, tok = engine(cfg, profile=profile)
+    st = Stream(fake)
+    eng.layer_step(1, tok, stream=st)
+    on = [s == st.cuda_stream for name, s in launches(fake) if name == "gemm"]
+    assert len(on) == 4 and on.count(False) == (0 if profile else 2)
+    eng.close()
