@@ -172,6 +172,37 @@ struct DeviceGuard {
     }
 };
 
+// Work of a call on a side stream, forked from the caller's stream and joined to
+// it again also when the call fails in between: the caller's next work uses the
+// same buffers and must not run beside what was left on the side.
+class SideBranch {
+public:
+    SideBranch(cudaStream_t main, cudaStream_t side, cudaEvent_t ev_fork, cudaEvent_t ev_join)
+        : main_(main), side_(side), fork_(ev_fork), join_(ev_join) {}
+    ~SideBranch() { join(); }
+    SideBranch(const SideBranch&) = delete;
+    SideBranch& operator=(const SideBranch&) = delete;
+    cudaError_t fork() {
+        cudaError_t e = cudaEventRecord(fork_, main_);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(side_, fork_, 0);
+        open_ = e == cudaSuccess;
+        return e;
+    }
+    cudaError_t join() {
+        if (!open_) return cudaSuccess;
+        open_ = false;
+        cudaError_t e = cudaEventRecord(join_, side_);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(main_, join_, 0);
+        if (e != cudaSuccess) cudaStreamSynchronize(side_);   // the host waits in the stream's place
+        return e;
+    }
+
+private:
+    cudaStream_t main_, side_;
+    cudaEvent_t fork_, join_;
+    bool open_ = false;
+};
+
 }  // namespace
 
 void tmoe::set_global_error(const std::string& msg) {
@@ -1100,11 +1131,10 @@ static trimmoe_status layer_step_impl(trimmoe_handle h, int layer, int T, trimmo
     // Already built for every layer at the start of the forward?
     const bool tabs_here = shared_tabs && !h->tabs_ready;
     const bool tabs_aside = tabs_here && c.M * E <= 256;
+    SideBranch tabs_branch(st, h->aux, h->ev_fork, h->ev_join);
     if (tabs_aside) {
-        e = cudaEventRecord(h->ev_fork, st);
-        if (e == cudaSuccess) e = cudaStreamWaitEvent(h->aux, h->ev_fork, 0);
+        e = tabs_branch.fork();
         if (e == cudaSuccess) e = launch_lookahead_shared(dp, n_depth, h->aux);
-        if (e == cudaSuccess) e = cudaEventRecord(h->ev_join, h->aux);
         if (e != cudaSuccess) return h->fail(TRIMMOE_ERR_CUDA, std::string("look-ahead tables: ") + cudaGetErrorString(e));
     }
     // Hidden rows for the router's TMA loads (128-token x 64-column boxes).
@@ -1120,7 +1150,7 @@ static trimmoe_status layer_step_impl(trimmoe_handle h, int layer, int T, trimmo
     if (has_attn) h->launches += 1;
     if (e != cudaSuccess) return h->fail(TRIMMOE_ERR_CUDA, std::string("router: ") + cudaGetErrorString(e));
     if (tabs_aside) {
-        e = cudaStreamWaitEvent(st, h->ev_join, 0);
+        e = tabs_branch.join();
         if (e != cudaSuccess) return h->fail(TRIMMOE_ERR_CUDA, std::string("look-ahead join: ") + cudaGetErrorString(e));
     }
     e = h->timed(K_DECIDE, st, [&] {
@@ -1206,12 +1236,10 @@ static trimmoe_status layer_step_impl(trimmoe_handle h, int layer, int T, trimmo
     // on the caller's stream: the times of launches that share the SMs would not
     // add up.
     const bool sh_aside = has_sh && c.profile == 0;
+    SideBranch sh_branch(st, h->aux, h->ev_fork, h->ev_join);
     if (has_sh) {
         cudaStream_t ss = sh_aside ? h->aux : st;
-        if (sh_aside) {
-            e = cudaEventRecord(h->ev_fork, st);
-            if (e == cudaSuccess) e = cudaStreamWaitEvent(ss, h->ev_fork, 0);
-        }
+        if (sh_aside) e = sh_branch.fork();
         if (e != cudaSuccess) return h->fail(TRIMMOE_ERR_CUDA, std::string("shared fork: ") + cudaGetErrorString(e));
         GemmLaunch s1 = g1;
         s1.ksplit = 1;
@@ -1247,8 +1275,6 @@ static trimmoe_status layer_step_impl(trimmoe_handle h, int layer, int T, trimmo
         h->n_gemm_up++;
         h->n_gemm_down++;
         h->launches += 2;
-        if (sh_aside) e = cudaEventRecord(h->ev_join, ss);
-        if (e != cudaSuccess) return h->fail(TRIMMOE_ERR_CUDA, std::string("shared join: ") + cudaGetErrorString(e));
     }
 
     e = h->timed(K_GEMM_UP, st, [&] {
@@ -1282,7 +1308,7 @@ static trimmoe_status layer_step_impl(trimmoe_handle h, int layer, int T, trimmo
     // (+ look-ahead tables, split-K finishes)
     h->launches += (fused ? 5 : 7) + (tabs_here ? 1 : 0) + (g1.ksplit > 1 ? 1 : 0) + (g2.ksplit > 1 ? 1 : 0);
     if (sh_aside) {
-        e = cudaStreamWaitEvent(st, h->ev_join, 0);
+        e = sh_branch.join();
         if (e != cudaSuccess) return h->fail(TRIMMOE_ERR_CUDA, std::string("shared join: ") + cudaGetErrorString(e));
     }
 

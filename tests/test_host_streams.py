@@ -88,3 +88,30 @@ def test_timed_launches_do_not_overlap(fake, profile):
     on = [s == st.cuda_stream for name, s in launches(fake) if name == "gemm"]
     assert len(on) == 4 and on.count(False) == (0 if profile else 2)
     eng.close()
+
+
+@pytest.mark.parametrize("what", ["launch", "record"])
+def test_failed_call_leaves_no_work_behind_on_the_side_stream(fake, what):
+    """Whichever launch or event record of a layer step fails, the caller's stream
+    (or the host) has waited for everything that the call put on the side stream:
+    the look-ahead tables beside the router, the shared expert's GEMMs beside the
+    routed ones."""
+    eng, tok = engine(shared_cfg(N=3, T=600))
+    st = Stream(fake)
+    eng.layer_step(1, tok, stream=st)
+    names = launches(fake)
+    side = [name for name, s in names if s != st.cuda_stream]
+    assert sorted(side) == ["gemm", "gemm", "tables"] and fake.fake_unordered(C.c_void_p(st.cuda_stream)) == 0
+    failures = 0
+    for n in range(len(names) + 1):
+        fake.fake_reset()
+        getattr(fake, f"fake_fail_{what}")(n)
+        try:
+            eng.layer_step(1, tok, stream=st)
+        except B.TrimmoeError:
+            failures += 1
+        assert fake.fake_unordered(C.c_void_p(st.cuda_stream)) == 0, (what, n)
+    assert failures == (len(names) if what == "launch" else 4)
+    fake.fake_reset()
+    eng.layer_step(1, tok, stream=st)
+    eng.close()
