@@ -295,8 +295,10 @@ struct trimmoe {
     float* la_scratch = nullptr;      // per-token look-ahead scratch of the decision kernel (shared-table layers)
     // Side stream, forked from and joined to the caller's within a layer: the
     // shared look-ahead tables (they depend only on the tables and the budget, so
-    // they are computed while the router runs) and the shared expert's GEMMs.
-    cudaStream_t aux = nullptr;
+    // they are computed while the router runs) and the shared expert's GEMMs.  One
+    // stream per priority of a caller's stream, made when a call first comes on it
+    // (the default priority's at create).
+    std::vector<std::pair<int, cudaStream_t>> aux;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     int rows_xp = 0;
 
@@ -372,6 +374,29 @@ struct trimmoe {
         allocs.push_back(q);
         *p = static_cast<T*>(q);
         return true;
+    }
+
+    // The side stream for calls on st; the default priority's if st's own cannot be
+    // had.
+    cudaStream_t aux_for(cudaStream_t st) {
+        int prio = 0;
+        if (st != nullptr && st != cudaStreamLegacy && st != cudaStreamPerThread &&
+            cudaStreamGetPriority(st, &prio) != cudaSuccess)
+            cudaGetLastError();
+        for (const auto& a : aux)
+            if (a.first == prio) return a.second;
+        // The caller may be capturing: making a stream is no part of the capture.
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        cudaStream_t s = nullptr;
+        const cudaError_t e = cudaStreamCreateWithPriority(&s, cudaStreamNonBlocking, prio);
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            return aux[0].second;
+        }
+        aux.push_back({prio, s});
+        return s;
     }
 
     cudaEvent_t get_event() {
@@ -826,7 +851,9 @@ extern "C" trimmoe_status trimmoe_create(const trimmoe_config* cfg, const trimmo
         // they must never hold NaN, so the buffer starts at zero.
         if (ce == cudaSuccess) ce = cudaMemset(h->vt, 0, h->vt_elems * sizeof(__nv_bfloat16));
     }
-    if (ce == cudaSuccess) ce = cudaStreamCreateWithFlags(&h->aux, cudaStreamNonBlocking);
+    cudaStream_t side = nullptr;
+    if (ce == cudaSuccess) ce = cudaStreamCreateWithFlags(&side, cudaStreamNonBlocking);
+    if (ce == cudaSuccess) h->aux.push_back({0, side});
     if (ce == cudaSuccess) ce = cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming);
     if (ce == cudaSuccess) ce = cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming);
     if (ce == cudaSuccess) ce = cudaMemset(h->ctr, 0, sizeof(DevCounters) * kCtrCopies);
@@ -1131,10 +1158,12 @@ static trimmoe_status layer_step_impl(trimmoe_handle h, int layer, int T, trimmo
     // Already built for every layer at the start of the forward?
     const bool tabs_here = shared_tabs && !h->tabs_ready;
     const bool tabs_aside = tabs_here && c.M * E <= 256;
-    SideBranch tabs_branch(st, h->aux, h->ev_fork, h->ev_join);
+    const bool sh_aside = has_sh && c.profile == 0;
+    const cudaStream_t side = tabs_aside || sh_aside ? h->aux_for(st) : nullptr;
+    SideBranch tabs_branch(st, side, h->ev_fork, h->ev_join);
     if (tabs_aside) {
         e = tabs_branch.fork();
-        if (e == cudaSuccess) e = launch_lookahead_shared(dp, n_depth, h->aux);
+        if (e == cudaSuccess) e = launch_lookahead_shared(dp, n_depth, side);
         if (e != cudaSuccess) return h->fail(TRIMMOE_ERR_CUDA, std::string("look-ahead tables: ") + cudaGetErrorString(e));
     }
     // Hidden rows for the router's TMA loads (128-token x 64-column boxes).
@@ -1233,12 +1262,11 @@ static trimmoe_status layer_step_impl(trimmoe_handle h, int layer, int T, trimmo
     // at a few tokens): Qwen-shaped, 8-token forwards of four layers 542 -> 478 us
     // alone and 261 -> 247 us with three streams, a layer of 700 tokens 308 -> 282
     // us, of 2000 387 -> 366 us, of 8192 831 -> 807 us.  With profiling they stay
-    // on the caller's stream: the times of launches that share the SMs would not
-    // add up.
-    const bool sh_aside = has_sh && c.profile == 0;
-    SideBranch sh_branch(st, h->aux, h->ev_fork, h->ev_join);
+    // on the caller's stream (sh_aside): the times of launches that share the SMs
+    // would not add up.
+    SideBranch sh_branch(st, side, h->ev_fork, h->ev_join);
     if (has_sh) {
-        cudaStream_t ss = sh_aside ? h->aux : st;
+        const cudaStream_t ss = sh_aside ? side : st;
         if (sh_aside) e = sh_branch.fork();
         if (e != cudaSuccess) return h->fail(TRIMMOE_ERR_CUDA, std::string("shared fork: ") + cudaGetErrorString(e));
         GemmLaunch s1 = g1;
@@ -1921,7 +1949,7 @@ extern "C" void trimmoe_destroy(trimmoe_handle h) {
     for (cudaEvent_t e : h->ev_free) cudaEventDestroy(e);
     if (h->ev_fork) cudaEventDestroy(h->ev_fork);
     if (h->ev_join) cudaEventDestroy(h->ev_join);
-    if (h->aux) cudaStreamDestroy(h->aux);
+    for (const auto& a : h->aux) cudaStreamDestroy(a.second);
     for (void* p : h->allocs) cudaFree(p);
     if (h->back_pinned) cudaFreeHost(h->back);
     else delete[] h->back;

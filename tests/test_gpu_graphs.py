@@ -177,3 +177,37 @@ def test_caller_capture_with_shared_expert():
         assert torch.equal(again[k], want[k]), k
     assert eng.stats()["status"] == 0
     eng.close()
+
+
+def test_capture_on_a_high_priority_stream():
+    """The first call on a high-priority stream may be inside the caller's capture:
+    the side stream of that priority is made there, and replays and plain calls
+    equal those on the default stream."""
+    import torch
+    cfg = small_cfg(name="prio", N=3, d=512, E=8, k=2, F=256, F_sh=384, T=300, M=8, H=3, seed=94)
+    eng, om, tables, small, experts = make_engine(cfg, T_max=300, theta=0.9, exit_bias=1.0)
+    init = eng.tokens_to_device(W.make_tokens(cfg))
+    want = {k: v.clone() for k, v in init.items()}
+    eng.layer_step(1, want)
+    eng.layer_step(2, want)
+    torch.cuda.synchronize()
+    work = {k: v.clone() for k, v in init.items()}
+    stream = torch.cuda.Stream(priority=-3)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=stream):
+        eng.layer_step(1, work, stream=stream)
+        eng.layer_step(2, work, stream=stream)
+    for replay in (True, True, False):
+        for k in work:
+            work[k].copy_(init[k])
+        torch.cuda.synchronize()
+        if replay:
+            g.replay()
+        else:
+            eng.layer_step(1, work, stream=stream)
+            eng.layer_step(2, work, stream=stream)
+        torch.cuda.synchronize()
+        for k in work:
+            assert torch.equal(work[k], want[k]), (k, replay)
+    assert eng.stats()["status"] == 0
+    eng.close()

@@ -115,3 +115,22 @@ def test_failed_call_leaves_no_work_behind_on_the_side_stream(fake, what):
     fake.fake_reset()
     eng.layer_step(1, tok, stream=st)
     eng.close()
+
+
+def test_side_stream_has_the_callers_priority(fake):
+    """The shared expert's GEMMs and the tables beside the router keep the
+    priority of the stream that the call came on, also when a program changes
+    between streams; the default streams have the default priority."""
+    eng, tok = engine(shared_cfg(N=3, T=600))
+    for ptr, prio in ((0x500, 0), (0x600, -5), (0x700, -2), (0x800, -5), (0x500, 0)):
+        st = Stream(fake, ptr, prio)
+        fake.fake_reset()
+        eng.layer_step(1, tok, stream=st)
+        side = [s for name, s in launches(fake) if s != ptr]
+        assert len(side) == 3 and {fake.fake_priority(C.c_void_p(s)) for s in side} == {prio}
+    for ptr in (0, 1, 2):       # the default stream, legacy and per thread
+        fake.fake_reset()
+        eng.layer_step(1, tok, stream=type("S", (), {"cuda_stream": ptr})())
+        side = [s for name, s in launches(fake) if s not in (ptr, None)]
+        assert len(side) == 3 and {fake.fake_priority(C.c_void_p(s)) for s in side} == {0}
+    eng.close()
