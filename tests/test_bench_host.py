@@ -124,3 +124,15 @@ def test_both_arms_print_the_same_config(bench_mod):
     a = bench_mod.config_dict(cfg, 1)
     assert a == bench_mod.config_dict(cfg, 1)
     assert a["workload"] == "mixtral" and a["T"] == 16384 and a["parallelism"] == "replicas1"
+
+
+def test_host_copy_bytes_count_what_is_copied(bench_mod):
+    """Every token array goes in; Dbar and pJ, which a forward only reads, do not
+    come back."""
+    import torch
+    T, d = 10, 256
+    host = dict(hidden=torch.zeros(T, d, dtype=torch.bfloat16), s=torch.zeros(T, dtype=torch.uint8),
+                Dhat=torch.zeros(T), Dbar=torch.zeros(T), pJ=torch.zeros(T), alive=torch.zeros(T, dtype=torch.uint8),
+                last_exec=torch.zeros(T, dtype=torch.uint8), xi_last=torch.zeros(T),
+                exit_layer=torch.zeros(T, dtype=torch.int16))
+    assert bench_mod.host_copy_bytes(host) == (T * (2 * d + 21), T * (2 * d + 13))
