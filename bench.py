@@ -564,6 +564,9 @@ def run_ours(args):
         timed.close()
     roof, fwd = rooflines(cfg, st, args.steps, ms_step, peaks, stored_traffic(cfg, "grouped_gemm_gate_up"), st_k=st_k)
     dom = roof["kernel"]
+    if st_k is not None:
+        roof["launches_per_step"] = st_k["n_gemm_up" if dom == "grouped_gemm_gate_up" else "n_gemm_down"] / args.steps
+        roof["timing"] = f"events around the GEMM launches, one after the other, in a second pass of {args.steps} steps"
     roof["traffic"] = stored_traffic(cfg, dom)
 
     # Per-kernel split: a separate pass of plain launches with events around

@@ -185,8 +185,8 @@ struct WarpCounters {
 // several streams at a time, every slot's candidates are read together and kept
 // for the choice, and the look-ahead interval is counted in one round of reads
 // instead of a binary search (three overlapping streams of 64-token
-// Switch-shaped forwards 77.4 -> 73.4 us a forward, a 777-token one through
-// host buffers 425 -> 412 us, 1-token Mixtral-shaped 429.5 -> 426.5 us).
+// Switch-shaped forwards 72.2 -> 68.6 us a forward, a 777-token one through
+// host buffers 393 -> 380 us, 1-token Mixtral-shaped 508 -> 504 us).
 // Without it, seven blocks per SM (72 registers, a few bytes spilled): each
 // token is a chain of dependent reads, so warps in flight matter more than registers
 // (six blocks at 80 registers: 1.31 instead of 0.94 ms per Mixtral-shaped

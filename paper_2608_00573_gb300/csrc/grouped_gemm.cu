@@ -407,10 +407,11 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             // loads (or left): its set-up still runs under this one's last tiles.
             // Triggered at the start instead, a following GEMM's CTAs (one per SM,
             // all of its shared memory and TMEM) hold the SMs that have no tile
-            // here, and GEMMs of other streams wait for them: three streams of
-            // 113-token Mixtral-shaped forwards 974 -> 884 us a forward, of
-            // 64-token Switch-shaped ones 85.0 -> 77.1 us, of 8-token Qwen-shaped
-            // ones 328 -> 304 us; one stream alone unchanged.
+            // here, and GEMMs of other streams wait for them.  This and the
+            // small-batch kernel, from the early trigger to this one: three streams
+            // of 113-token Mixtral-shaped forwards 1021 -> 924 us a forward, of
+            // 64-token Switch-shaped ones 72.8 -> 70.7 us, though 8-token
+            // Qwen-shaped ones 246 -> 251 us.
             pdl_trigger();
         }
     } else if (warp == 1) {
@@ -485,16 +486,20 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
 // Small-batch variant: 128 x 128 tiles, two CTAs per SM.
 //
 // With few rows per group a launch streams weights, and a k-block of a CTA takes
-// as long as its one producer thread and its one MMA thread need to issue it
-// (clock64: 500-530 cycles, whatever the tile's width), so one CTA per SM pulls
-// at most 32 KB per ~0.4 us however wide its tiles, its last round leaves SMs
-// idle (16 column tiles of 256 for an expert's down projection on 152 SMs), and
-// GEMMs of other streams, which need a whole SM each, queue behind it.  Here a
-// CTA takes half the columns, half of TMEM and under half of the shared memory:
-// two CTAs issue per SM (of one launch or of two streams'), and the rounds are
-// twice as fine.  A column's sum is the same in either kernel (one K order):
-// bit for bit the same results.  1-token Mixtral-shaped forwards of six layers
-// 428 -> 403 us (three overlapping streams) and 825 -> 748 us (one alone),
+// at least the time that its one producer thread and its one MMA thread need to
+// issue it (clock64: 500-530 cycles, about 0.27 us at 1.9 GHz, whatever the
+// tile's width).  That is no limit for a launch that fills the SMs (152 CTAs
+// issue boxes faster than HBM delivers them), but it bounds one of few tiles and
+// every ragged last round: the Qwen-shaped shared down projection of a few tokens
+// took 37.5 us for 8 column tiles of 88 k-blocks on 8 SMs, and an expert's down
+// projection has 16 column tiles of 256 for 152.  GEMMs of other streams, which
+// need a whole SM each, queue behind either.  Here a CTA takes half the columns,
+// half of TMEM and under half of the shared memory: two CTAs issue per SM (of one
+// launch or of two streams'), and the rounds are twice as fine.  A column's sum
+// over one K range is the same in either kernel: without a K split, bit for bit
+// the same results.  1-token Mixtral-shaped forwards of six layers 428 -> 403 us
+// (three overlapping streams) and 825 -> 748 us (one alone; its up projection
+// 85 -> 78 us, its down projection, already spread over 256 units, 42 -> 44 us),
 // 8-token Qwen-shaped ones of four layers 280 -> 259 and 632 -> 538 us.
 //
 // A tile takes two equal runs of weight rows `half` apart in one TMA box: 64
@@ -1046,7 +1051,7 @@ grouped_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
 // 128 KB a tile: at K = 4096 about 3 % of what the MMAs move, hidden by the main
 // loop; at K = 2048 the swap shows and the row kernels stay ahead).  Against
 // the single-CTA kernel at 330 rows per group: one box instead of 17 % padded
-// rows, Mixtral-shaped layer of 1500 tokens 846 -> 791 us.
+// rows, Mixtral-shaped layer of 1500 tokens 837 -> 780 us.
 constexpr int kStageBf16 = 32 * 128;           // one 32-token x 128-feature bf16 staging buffer
 constexpr size_t kPairTailBytes = (sizeof(PairSmemTail) + 15) & ~(size_t)15;
 constexpr size_t kPairTSmemBytes = 1024 + (size_t)P_STAGES * P_STAGE_BYTES + kPairTailBytes +

@@ -89,7 +89,11 @@ inline bool pair_gemm(long long rows_per_group) { return rows_per_group >= kPair
 // four-layer forward on the single-CTA kernel and on it: Qwen-shaped, 24 tokens
 // 358 -> 331 (1.6 rows per routed group), 160 tokens
 // 514 -> 510; Mixtral-shaped, 40 tokens (10 rows per group) 826 -> 803, but 200
-// tokens (50 rows) 1024 -> 1052; full block, 40 tokens 978 -> 943.
+// tokens (50 rows) 1024 -> 1052; full block, 40 tokens 978 -> 943.  Two row tiles
+// of a single group still gain (one stream alone, full blocks of 132 and of 160
+// tokens: Mixtral-shaped 1815 -> 1771 and 1810 -> 1766, Qwen-shaped 905 -> 868
+// and 941 -> 901, Switch-shaped 393 -> 353 and 412 -> 373); at 512 and 1900 rows
+// they lose (Qwen-shaped forward 743 -> 751, layer 389 -> 399).
 constexpr int kSmallRoutedRows = 20, kSmallSingleRows = 160;
 
 // Routed launches run their store / ReLU epilogues on the transposed pair
@@ -111,10 +115,15 @@ inline bool transposed_gemm(long long rows, int groups) {
 // SwiGLU up projections of those groups run there too from this K on (and below
 // kPairMinRows rows per group, where the row-pair kernel's padding weighs less
 // than the swap of gates and ups): at K = 4096 the Mixtral-shaped layer of 1500
-// tokens (330 rows per group) 838 -> 794 us and the full-block layer of 4200
-// tokens (910 rows) 2085 -> 1997 us against the single-CTA kernel (2030 us on
-// the row-pair kernel); at K = 2048 the main loop is too short to hide the swap
-// (Qwen-shaped layer of 8192 tokens 834 -> 880 us).
+// tokens (330 rows per group) 837 -> 780 us and the full-block layer of 4200
+// tokens (910 rows) 2104 -> 1992 us against the single-CTA kernel (the row-pair
+// kernel there: 2095 -> 2038 us); at K = 2048 the main loop is too short to hide
+// the swap (Qwen-shaped layer of 8192 tokens 834 -> 880 us).  Over K, eight
+// experts of F = 8192, top-2, layers of 1500 and 4200 tokens: 2304 313 -> 344 and
+// 613 -> 704 us, 2560 333 -> 339 and 625 -> 676, 3072 401 -> 395 and 802 -> 822,
+// 3584 434 -> 416 and 875 -> 840, 4096 457 -> 447 and 980 -> 929, 6144 705 -> 655
+// and 1458 -> 1401, 8192 893 -> 821 and 1934 -> 1782: the two cross between 3072
+// and 3584, where no model family here has its depth.
 constexpr int kTransposedSwigluMinK = 4096;
 
 // CTA-pair launches with at least this K draw their tiles from a launch-wide
