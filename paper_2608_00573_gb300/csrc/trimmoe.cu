@@ -862,7 +862,10 @@ extern "C" trimmoe_status trimmoe_create(const trimmoe_config* cfg, const trimmo
     }
     cudaStream_t side = nullptr;
     if (ce == cudaSuccess) ce = cudaStreamCreateWithFlags(&side, cudaStreamNonBlocking);
-    if (ce == cudaSuccess) h->aux.push_back({0, side});
+    if (ce == cudaSuccess) {
+        h->aux.reserve(16);      // more than there are priorities: a call never reallocates it
+        h->aux.push_back({0, side});
+    }
     if (ce == cudaSuccess) ce = cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming);
     if (ce == cudaSuccess) ce = cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming);
     if (ce == cudaSuccess) ce = cudaMemset(h->ctr, 0, sizeof(DevCounters) * kCtrCopies);
